@@ -1865,6 +1865,12 @@ std::string generate_source(const std::vector<Pattern> &pats, const std::vector<
             << "(const ExaTile* __restrict__ tiles, const int ntiles, const ExaPM* __restrict__ pms,"
                " const double* __restrict__ x, const double* __restrict__ y, const double* __restrict__ th,"
                " const double sigma, const ExaOut o, const ExaStructOut so, const int pfd) {\n";
+        // Launched with programmatic stream serialization: the next kernel's blocks may be scheduled while
+        // this one drains, and nothing here reads inputs or writes outputs before the kernels ahead of
+        // it have completed.
+        if (m != M_STRUCT)
+            src << "  asm volatile(\"griddepcontrol.launch_dependents;\" ::: \"memory\");\n"
+                   "  asm volatile(\"griddepcontrol.wait;\" ::: \"memory\");\n";
         if (objred) src << "  __shared__ double red[EXA_BLOCK / 32];\n";
         if (m != M_STRUCT)
             src << "  __shared__ double stage[EXA_BLOCK * " << smax << "];\n"

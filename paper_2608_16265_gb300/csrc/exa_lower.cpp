@@ -1867,10 +1867,10 @@ std::string generate_source(const std::vector<Pattern> &pats, const std::vector<
                " const double sigma, const ExaOut o, const ExaStructOut so, const int pfd) {\n";
         // Launched with programmatic stream serialization: the next kernel's blocks may be scheduled while
         // this one drains, and nothing here reads inputs or writes outputs before the kernels ahead of
-        // it have completed.
+        // it have completed (the input pointers pass through the wait, so no load moves ahead of it).
         if (m != M_STRUCT)
             src << "  asm volatile(\"griddepcontrol.launch_dependents;\" ::: \"memory\");\n"
-                   "  asm volatile(\"griddepcontrol.wait;\" ::: \"memory\");\n";
+                   "  asm volatile(\"griddepcontrol.wait;\" : \"+l\"(x), \"+l\"(y), \"+l\"(th) : : \"memory\");\n";
         if (objred) src << "  __shared__ double red[EXA_BLOCK / 32];\n";
         if (m != M_STRUCT)
             src << "  __shared__ double stage[EXA_BLOCK * " << smax << "];\n"

@@ -22,8 +22,12 @@
 namespace exa_red {
 
 // Waits until the kernels this one depends on have completed and their writes are visible (no-op
-// for an ordinary launch); lets the next kernel's blocks be scheduled.
-static __device__ __forceinline__ void wait_inputs() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
+// for an ordinary launch), and returns src: loads through the returned pointer cannot be moved ahead of
+// the wait, whatever kind of load they are.  allow_next lets the next kernel's blocks be scheduled.
+static __device__ __forceinline__ const double *wait_inputs(const double *src) {
+    asm volatile("griddepcontrol.wait;" : "+l"(src) : : "memory");
+    return src;
+}
 static __device__ __forceinline__ void allow_next() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
 
 enum Kind {
@@ -74,10 +78,10 @@ static __device__ __forceinline__ void perm_job(const Job &j, int blk) {
 #pragma unroll
         for (int u = 0; u < ILP; u++) p[u] = THREADS * u < left ? __ldg(perm + THREADS * u) : ELSEWHERE;
     }
-    wait_inputs();
+    const double *src = wait_inputs(j.src);
     double v[ILP];
 #pragma unroll
-    for (int u = 0; u < ILP; u++) v[u] = p[u] >= 0 ? __ldcg(j.src + p[u]) : 0.0;
+    for (int u = 0; u < ILP; u++) v[u] = p[u] >= 0 ? __ldcg(src + p[u]) : 0.0;
     double *dst = j.dst + i0;
 #pragma unroll
     for (int u = 0; u < ILP; u++)
@@ -93,7 +97,7 @@ static __device__ __forceinline__ void seg_job(const Job &j, int blk, double *bu
     const int lane = threadIdx.x & 31;
     const unsigned s0 = ((unsigned)blk * (THREADS / 32) + (threadIdx.x >> 5)) * (32 * G);
     if (s0 >= (unsigned)j.n) {
-        wait_inputs();
+        wait_inputs(j.src);
         return;
     }
     double *b = buf + (threadIdx.x >> 5) * PIECE;
@@ -108,14 +112,14 @@ static __device__ __forceinline__ void seg_job(const Job &j, int blk, double *bu
     }
 #pragma unroll
     for (int u = 0; u < PIECE / 32; u++) p[u] = beg + lane + 32 * u < end ? __ldg(j.perm + beg + lane + 32 * u) : -1;
-    wait_inputs();
+    const double *src = wait_inputs(j.src);
     double acc[G];
 #pragma unroll
     for (int g = 0; g < G; g++) acc[g] = j.add && 32 * g < left ? j.dst[__ldg(j.row + s0 + lane + 32 * g)] : 0.0;
     for (int c0 = beg;;) {
 #pragma unroll
         for (int u = 0; u < PIECE / 32; u++)
-            if (p[u] >= 0) b[lane + 32 * u] = __ldcg(j.src + p[u]);
+            if (p[u] >= 0) b[lane + 32 * u] = __ldcg(src + p[u]);
         __syncwarp();
         const int c1 = min(c0 + PIECE, end);
 #pragma unroll
@@ -193,10 +197,10 @@ static __global__ void __launch_bounds__(THREADS, 6) k_reduce(const __grid_const
         break;
     case WSEG: case CSUM: {
         const int s = blk * (THREADS / 32) + w;
-        wait_inputs();
+        const double *src = wait_inputs(j.src);
         if (s >= j.n) break;
         const int *r = j.kind == CSUM ? j.ptr + s : j.ptr + 2 * (long long)s;
-        const double t = warp_sum(strided_sum(j.src, j.kind == CSUM ? nullptr : j.perm, __ldg(r), __ldg(r + 1), lane, 32));
+        const double t = warp_sum(strided_sum(src, j.kind == CSUM ? nullptr : j.perm, __ldg(r), __ldg(r + 1), lane, 32));
         if (lane == 0) {
             double *d = j.dst + __ldg(j.row + s);
             *d = j.add ? *d + t : t;
@@ -204,21 +208,21 @@ static __global__ void __launch_bounds__(THREADS, 6) k_reduce(const __grid_const
         break;
     }
     case CHUNK: {
-        wait_inputs();
-        const double t = block_sum(strided_sum(j.src, j.perm, __ldg(j.ptr + 2 * (long long)blk), __ldg(j.ptr + 2 * (long long)blk + 1), threadIdx.x, THREADS), buf);
+        const double *src = wait_inputs(j.src);
+        const double t = block_sum(strided_sum(src, j.perm, __ldg(j.ptr + 2 * (long long)blk), __ldg(j.ptr + 2 * (long long)blk + 1), threadIdx.x, THREADS), buf);
         if (threadIdx.x == 0) j.dst[blk] = t;
         break;
     }
     case OBJ: {
-        wait_inputs();
-        const double t = block_sum(strided_sum(j.src, nullptr, 0, j.n, threadIdx.x, THREADS), buf);
+        const double *src = wait_inputs(j.src);
+        const double t = block_sum(strided_sum(src, nullptr, 0, j.n, threadIdx.x, THREADS), buf);
         if (threadIdx.x == 0) j.dst[0] = t;
         break;
     }
     default: {  // FILL: 32 positions per thread, one mask word
         const long long word = j.lo / 32 + (long long)blk * THREADS + threadIdx.x;
         unsigned keep = word * 32 < j.n ? __ldg((const unsigned *)j.ptr + word) : 0xffffffffu;
-        wait_inputs();
+        wait_inputs(nullptr);
         // a warp writes its 1024 positions as 32 coalesced rows
         for (int r = 0; r < 32; r++) {
             const unsigned k = __shfl_sync(0xffffffffu, keep, r);
@@ -234,7 +238,7 @@ static __global__ void __launch_bounds__(THREADS, 6) k_reduce(const __grid_const
 static __global__ void __launch_bounds__(1024) k_obj_final(const double *part, int n, double *f) {
     __shared__ double buf[32];
     allow_next();
-    wait_inputs();
+    part = wait_inputs(part);
     const double t = block_sum(strided_sum(part, nullptr, 0, n, threadIdx.x, blockDim.x), buf);
     if (threadIdx.x == 0) f[0] = t;
 }

@@ -32,6 +32,8 @@
         long long gbase[16];      /* per pattern: first gradient-buffer slot */                     \
         long long abase[16];      /* per pattern: first augmentation-buffer entry */                \
         long long hcbase;         /* first slot of the group's compressed Hessian sums */           \
+        long long tbase;          /* first slot of the group's J^T w terms: [symbol][instance] */   \
+        long long ubase;          /* first slot of the group's H v terms: [symbol][instance] */     \
         int grp;                  /* group id */                                                    \
         int member;               /* batch member */                                                \
     };                                                                                              \
@@ -52,9 +54,11 @@
         const int *hmap;          /* Hessian COO slot -> CSC position */                            \
         double *hcomp;            /* if set: per-instance sums of the group's equal Hessian pairs */\
         int *status;              /* device fault word (bounds) */                                  \
+        const double *v;          /* products: the vector */                                        \
+        double *prod;             /* products: J^T w or H v terms per instance and group symbol */  \
     };                                                                                              \
     struct ExaStructOut {                                                                           \
-        int *jrow, *jcol, *hrow, *hcol, *gvar, *arow, *hcrow, *hccol;                               \
+        int *jrow, *jcol, *hrow, *hcol, *gvar, *arow, *hcrow, *hccol, *tvar, *uvar;                 \
         int *status;                                                                                \
     };                                                                                              \
     struct ExaTask {              /* one item of the fused step's work queue */                     \
@@ -87,13 +91,15 @@ namespace exa {
 // (gradient slots / Jacobian), second order (Hessian), all of them, all but second order, and the
 // structure pass that writes the COO rows and columns.  The Hessian-producing kinds come in three
 // compile-time variants: COO slots (M_HESS, M_ALL), the group-compressed sums used for the CSC
-// (..._C), or both (..._B).
+// (..._C), or both (..._B).  The products J v, J^T w and H v contract each instance's derivatives with
+// the vector where they are formed (M_JPROD, M_JTPROD, M_HPROD; a module of their own).
 enum Mode { M_OBJ = 0, M_CON, M_GRAD, M_JAC, M_HESS, M_ALL, M_FIRST, M_STRUCT,
-            M_HESS_C, M_HESS_B, M_ALL_C, M_ALL_B, M_COUNT };
-inline bool mode_hess(int m) { return m == M_HESS || m == M_ALL || m >= M_HESS_C; }
+            M_HESS_C, M_HESS_B, M_ALL_C, M_ALL_B, M_JPROD, M_JTPROD, M_HPROD, M_COUNT };
+inline bool mode_prod(int m) { return m >= M_JPROD; }
+inline bool mode_hess(int m) { return m == M_HESS || m == M_ALL || (m >= M_HESS_C && m <= M_ALL_B); }
 inline bool mode_all(int m) { return m == M_ALL || m == M_ALL_C || m == M_ALL_B; }
 inline bool mode_hess_coo(int m) { return m == M_HESS || m == M_ALL || m == M_HESS_B || m == M_ALL_B; }
-inline bool mode_hess_comp(int m) { return m >= M_HESS_C; }
+inline bool mode_hess_comp(int m) { return m >= M_HESS_C && m <= M_ALL_B; }
 extern const char *const kModeName[M_COUNT];
 
 struct VNode { int op, a, b; long long iv; double fv; };
@@ -131,6 +137,7 @@ struct Group {
     // same (row, col) for every instance), summed per instance; each entry lists (position, slot)
     std::vector<std::vector<std::pair<int, int>>> hc;
     std::vector<std::pair<int, int>> hc_sym;  // group symbol pair of each compressed slot
+    std::vector<int> tsym, usym;  // group symbols of the constraints' first-order slots / of the Hessian
 };
 
 // Unifies the symbols of a group's patterns: equal index expressions (columns compared as group
@@ -171,6 +178,8 @@ struct CodegenOptions {
     // and the step's reductions taken from one work queue (ExaStep).  Excludes staging, prefetch
     // and warp sets.
     bool fused_step = false;
+    // the module of the product kernels instead of all others (block only; no other choice applies)
+    bool products = false;
 };
 // The warp sets of group g in kernel kind `mode` (positions in g.pats per set, in order): one set
 // with every active pattern, or `lanes` contiguous subsets of about equal outputs.

@@ -37,7 +37,7 @@ namespace exa {
 #define EXA_STR(...) EXA_STR2(__VA_ARGS__)
 const char *const kDeviceStructs = EXA_STR(EXA_DEVICE_STRUCTS);
 const char *const kModeName[M_COUNT] = {"obj", "con", "grad", "jac", "hess", "all", "first", "struct",
-                                        "hess_c", "hess_b", "all_c", "all_b"};
+                                        "hess_c", "hess_b", "all_c", "all_b", "jprod", "jtprod", "hprod"};
 
 static bool is_unary(int op) { return op >= EXA_V_NEG && op <= EXA_V_EXP2; }
 static bool is_binary(int op) { return op >= EXA_V_ADD && op <= EXA_V_HYPOT; }
@@ -792,6 +792,234 @@ static void build_graph(const Pattern &p, const InputMap &im, Graph &g, PatternG
         }
 }
 
+// ------------------------------------------------------------------ products (FP64)
+// J v, J^T w and H v of one group instance, formed on the group's shared graph instead of from the
+// derivative entries: J v by forward differentiation of every pattern's value in direction v (inputs
+// 'V', per group symbol), J^T w as the gradient of sum w_p f_p (inputs 'W', per pattern position) by one
+// reverse pass over all patterns, H v as the forward derivative of that gradient.  The FP64 pipe binds
+// these kernels, so the reverse pass keeps adjoints as sums of products and takes out the factors that
+// all their terms share before it goes on: the flow patterns of a branch, w_p v_f v_t (g_p cos + b_p sin),
+// give v_f v_t (cos (sum w_p g_p) + ...) with two multiply-adds per pattern.  (Mixed precision contracts
+// the FP32-rounded entries themselves, so that its products are those of its Jacobian and Hessian.)
+struct ProdGraph {
+    std::vector<int> jv;      // per position: the row's product (-1: not a constraint)
+    std::vector<int> jt, hv;  // per entry of the group's tsym / usym (-1: zero)
+};
+
+class Products {
+    Graph &g;
+    std::map<int, bool> dep_;
+    std::map<int, int> tan_;
+    typedef std::map<std::vector<int>, double> Terms;  // sorted factors -> coefficient
+
+    bool dep(int n) {  // depends on x
+        auto it = dep_.find(n);
+        if (it != dep_.end()) return it->second;
+        const SN s = g.n[n];
+        const bool d = s.op == S_IN ? s.ikind == 'X' : (s.a >= 0 && dep(s.a)) || (s.b >= 0 && dep(s.b));
+        return dep_[n] = d;
+    }
+    int one() { return g.lit(1.0, PD); }
+    // partial derivatives of node n for its operands, as build_graph forms them
+    int partial(int n, int which) {
+        const SN s = g.n[n];
+        const int a = s.a, b = s.b;
+        switch (s.op) {
+        case S_NEG: return g.lit(-1.0, PD);
+        case S_ADD: return one();
+        case S_SUB: return which ? g.lit(-1.0, PD) : one();
+        case S_MUL: return which ? a : b;
+        case S_DIV: {
+            const int r = g.div(one(), b);
+            return which ? g.neg(g.mul(n, r)) : r;
+        }
+        case S_EXP: return n;
+        case S_LOG: return g.div(one(), a);
+        case S_SIN: return g.fn(S_COS, a);
+        case S_COS: return g.neg(g.fn(S_SIN, a));
+        case S_SQRT: return g.div(g.lit(0.5, PD), n);
+        case S_TAN: return g.add(one(), g.mul(n, n));
+        case S_TANH: return g.sub(one(), g.mul(n, n));
+        case S_ATAN: return g.div(one(), g.add(one(), g.mul(a, a)));
+        case S_SINH: return g.fn(S_COSH, a);
+        case S_COSH: return g.fn(S_SINH, a);
+        case S_ASIN: case S_ACOS: {
+            const int r = g.div(one(), g.fn(S_SQRT, g.sub(one(), g.mul(a, a))));
+            return s.op == S_ASIN ? r : g.neg(r);
+        }
+        case S_LOG1P: return g.div(one(), g.add(one(), a));
+        case S_EXPM1: return g.fn(S_EXP, a);
+        case S_LOG2: case S_LOG10:
+            return g.div(one(), g.mul(a, g.lit(s.op == S_LOG2 ? 0.69314718055994531 : 2.3025850929940457, PD)));
+        case S_EXP2: return g.mul(n, g.lit(0.69314718055994531, PD));
+        case S_POW: return which ? g.mul(n, g.fn(S_LOG, a)) : g.mul(b, g.div(n, a));
+        case S_ATAN2: {
+            const int r = g.add(g.mul(a, a), g.mul(b, b));
+            return which ? g.neg(g.div(a, r)) : g.div(b, r);
+        }
+        case S_HYPOT: return g.div(which ? b : a, n);
+        default: return -1;
+        }
+    }
+    // coefficient and sorted factors of a node seen as a product
+    void factors(int n, double &c, std::vector<int> &f) {
+        const SN s = g.n[n];
+        if (s.op == S_NEG) { c = -c; factors(s.a, c, f); }
+        else if (s.op == S_MUL) { factors(s.a, c, f); factors(s.b, c, f); }
+        else if (s.op == S_LIT) c *= s.lit;
+        else f.push_back(n);
+    }
+    // the product of the factors, by products that the graph has already where there are any
+    int product(std::vector<int> f) {
+        if (f.empty()) return one();
+        int node, sign;
+        if (f.size() > 1 && g.find_prod(PD, f, node, sign)) return sign < 0 ? g.neg(node) : node;
+        while (f.size() > 1) {
+            size_t bi = 0, bj = 1;
+            for (size_t i = 0; i < f.size(); i++)
+                for (size_t j = i + 1; j < f.size(); j++)
+                    if (g.has(S_MUL, PD, std::min(f[i], f[j]), std::max(f[i], f[j]))) { bi = i; bj = j; i = f.size() - 1; break; }
+            const int m = g.mul(f[bi], f[bj]);
+            f.erase(f.begin() + bj);
+            f.erase(f.begin() + bi);
+            f.insert(f.begin(), m);
+        }
+        return f[0];
+    }
+    int scaled(double c, int n) {
+        return c < 0 ? g.neg(scaled(-c, n)) : c == 1.0 ? n : g.mul(g.lit(c, PD), n);
+    }
+    // sum of the terms as coefficient x (common factors) x (rest), the rest a node
+    void collapse(const Terms &t, double &c, std::vector<int> &common) {
+        common.clear();
+        c = 1.0;
+        if (t.size() == 1) {
+            c = t.begin()->second;
+            common = t.begin()->first;
+            return;
+        }
+        bool first = true;
+        for (auto &kv : t) {
+            if (first) common = kv.first;
+            else {
+                std::vector<int> x;
+                std::set_intersection(common.begin(), common.end(), kv.first.begin(), kv.first.end(), std::back_inserter(x));
+                common = x;
+            }
+            first = false;
+        }
+        int sum = -1;
+        for (auto &kv : t) {
+            std::vector<int> rest;
+            std::set_difference(kv.first.begin(), kv.first.end(), common.begin(), common.end(), std::back_inserter(rest));
+            const int p = scaled(kv.second, product(rest));
+            sum = sum < 0 ? p : g.add(sum, p);
+        }
+        factors(sum, c, common);
+        std::sort(common.begin(), common.end());
+    }
+    int value(const Terms &t) {
+        double c;
+        std::vector<int> f;
+        collapse(t, c, f);
+        return scaled(c, product(f));
+    }
+
+    // the derivative of node n in direction v as a sum of products: sums are kept open, so that the
+    // factors all their terms share come out at the top
+    Terms tangent_terms(int n) {
+        Terms r;
+        if (!dep(n)) return r;
+        const SN s = g.n[n];
+        if (s.op == S_IN) {
+            r[{g.input('V', s.iid, PD)}] = 1.0;
+            return r;
+        }
+        for (int which = 0; which < 2; which++) {
+            const int k = which ? s.b : s.a;
+            if (k < 0 || !dep(k)) continue;
+            const Terms t = tangent_terms(k);
+            if (t.empty()) continue;
+            if (s.op == S_ADD || s.op == S_SUB || s.op == S_NEG) {
+                const double sign = s.op == S_NEG || (s.op == S_SUB && which) ? -1.0 : 1.0;
+                for (auto &kv : t) r[kv.first] += sign * kv.second;
+            } else {
+                double c;
+                std::vector<int> f;
+                collapse(t, c, f);
+                factors(partial(n, which), c, f);
+                std::sort(f.begin(), f.end());
+                r[f] += c;
+            }
+        }
+        for (auto it = r.begin(); it != r.end();) it = it->second == 0.0 ? r.erase(it) : std::next(it);
+        return r;
+    }
+
+  public:
+    explicit Products(Graph &graph) : g(graph) {}
+
+    // derivative of node n in direction v (-1: zero)
+    int tangent(int n) {
+        auto it = tan_.find(n);
+        if (it != tan_.end()) return it->second;
+        const Terms t = tangent_terms(n);
+        return tan_[n] = t.empty() ? -1 : value(t);
+    }
+    // gradient over group symbols of the sum of w_p value_p over the given (position, value) pairs
+    std::map<int, int> gradient(const std::vector<std::pair<int, int>> &values) {
+        std::map<int, Terms, std::greater<int>> adj;
+        for (auto &pv : values)
+            if (dep(pv.second)) adj[pv.second][{g.input('W', pv.first, PD)}] += 1.0;
+        std::map<int, int> grad;
+        while (!adj.empty()) {
+            const int n = adj.begin()->first;  // operands have smaller ids: all its terms are there
+            Terms t = adj.begin()->second;
+            adj.erase(adj.begin());
+            for (auto it = t.begin(); it != t.end();) it = it->second == 0.0 ? t.erase(it) : std::next(it);
+            if (t.empty()) continue;
+            const SN s = g.n[n];
+            if (s.op == S_IN) {
+                grad[s.iid] = value(t);
+                continue;
+            }
+            double c;
+            std::vector<int> f;
+            collapse(t, c, f);
+            if (f.size() > 4) f = {product(f)};
+            for (int which = 0; which < 2; which++) {
+                const int k = which ? s.b : s.a;
+                if (k < 0 || !dep(k)) continue;
+                double ck = c;
+                std::vector<int> fk = f;
+                factors(partial(n, which), ck, fk);
+                std::sort(fk.begin(), fk.end());
+                adj[k][fk] += ck;
+            }
+        }
+        return grad;
+    }
+};
+
+static ProdGraph build_products(const std::vector<Pattern> &pats, const Group &grp, Graph &g,
+                                const std::vector<PatternGraph> &PG) {
+    ProdGraph r;
+    Products P(g);
+    std::vector<std::pair<int, int>> con, curved;
+    r.jv.assign(grp.pats.size(), -1);
+    for (size_t pos = 0; pos < grp.pats.size(); pos++) {
+        const Pattern &p = pats[grp.pats[pos]];
+        if (p.nh() > 0) curved.push_back({(int)pos, PG[pos].value});
+        if (p.kind == EXA_OBJ) continue;
+        con.push_back({(int)pos, PG[pos].value});
+        r.jv[pos] = P.tangent(PG[pos].value);
+    }
+    std::map<int, int> gt = P.gradient(con), gh = P.gradient(curved);
+    for (int s : grp.tsym) r.jt.push_back(gt.count(s) ? gt[s] : -1);
+    for (int s : grp.usym) r.hv.push_back(gh.count(s) ? P.tangent(gh[s]) : -1);
+    return r;
+}
+
 }  // namespace
 
 // ------------------------------------------------------------------ group symbols
@@ -840,13 +1068,19 @@ void finalize_group(Group &g, const std::vector<Pattern> &pats) {
             g.hc[r.first->second].push_back({(int)pos, j});
         }
     }
+    std::set<int> t, u;
+    for (size_t pos = 0; pos < g.pats.size(); pos++)
+        if (pats[g.pats[pos]].kind != EXA_OBJ) t.insert(g.sym[pos].begin(), g.sym[pos].end());
+    for (auto &pr : g.hc_sym) u.insert({pr.first, pr.second});
+    g.tsym.assign(t.begin(), t.end());
+    g.usym.assign(u.begin(), u.end());
 }
 
 bool pattern_in_mode(const Pattern &p, Mode m) {
     switch (m) {
     case M_OBJ: case M_GRAD: return p.kind == EXA_OBJ;
-    case M_CON: case M_JAC: return p.kind != EXA_OBJ;
-    case M_HESS: case M_HESS_C: case M_HESS_B: return p.nh() > 0;
+    case M_CON: case M_JAC: case M_JPROD: case M_JTPROD: return p.kind != EXA_OBJ;
+    case M_HESS: case M_HESS_C: case M_HESS_B: case M_HPROD: return p.nh() > 0;
     default: return true;
     }
 }
@@ -855,7 +1089,7 @@ std::vector<std::vector<int>> group_sets(const std::vector<Pattern> &pats, const
     std::vector<int> act;
     for (size_t pos = 0; pos < g.pats.size(); pos++)
         if (pattern_in_mode(pats[g.pats[pos]], mode)) act.push_back((int)pos);
-    if (lanes < 2 || (int)act.size() < 2 || mode == M_STRUCT || mode_hess_comp(mode)) return {act};
+    if (lanes < 2 || (int)act.size() < 2 || mode == M_STRUCT || mode_hess_comp(mode) || mode_prod(mode)) return {act};
     // two contiguous subsets, the cut that best balances the outputs (values, first- and
     // second-order slots) of the two sides
     auto cost = [&](int pos) { const Pattern &p = pats[g.pats[pos]]; return 1 + p.nj() + p.nh(); };
@@ -879,6 +1113,7 @@ struct Emitter {
     const Graph &g;
     const std::vector<PatternGraph> &PG;  // per position in the group
     const CodegenOptions &opt;
+    const ProdGraph *prod = nullptr;  // FP64 products (null: contract the derivative entries)
     std::ostringstream os;
     std::string pf_text;  // prefetch functions of the last function() (opt.prefetch > 0)
     // shared-memory staging (opt.stage): the last function()'s stage function and its 8- and
@@ -1002,12 +1237,12 @@ struct Emitter {
                     std::string cn = ci >= 0 ? "t" + std::to_string(ci) : t + "_c";
                     os << "  " << T << " " << sn << ", " << cn << ";\n";
                     if (red) os << "  exa_sincos_red(" << A() << ", &" << sn << ", &" << cn << ");\n";
-                    else os << "  " << (s.prec == PF ? "sincosf(" : "exa_sincos64(") << A() << ", &" << sn << ", &" << cn << ");\n";
+                    else os << "  " << (s.prec == PF ? "sincosf(" : opt.products ? "exa_sincos64_warp(" : "exa_sincos64(") << A() << ", &" << sn << ", &" << cn << ");\n";
                     if (si >= 0) name[si] = sn;
                     if (ci >= 0) name[ci] = cn;
                 } else if (s.prec == PD) {  // one of the pair: the other result is dead code
                     os << "  double " << t << "_s, " << t << "_c;\n"
-                       << "  exa_sincos64(" << A() << ", &" << t << "_s, &" << t << "_c);\n"
+                       << "  exa_sincos64" << (opt.products ? "_warp" : "") << "(" << A() << ", &" << t << "_s, &" << t << "_c);\n"
                        << "  const double " << t << " = " << t << (s.op == S_SIN ? "_s" : "_c") << ";\n";
                 } else {
                     os << "  const " << T << " " << t << " = " << fname(s.op, s.prec) << "(" << A() << ");\n";
@@ -1026,7 +1261,10 @@ struct Emitter {
         const bool mixed = opt.precision == EXA_MIXED_FP32;
         const char *W = mixed ? "float" : "double";
         const bool all = mode_all(mode) || mode == M_FIRST;
-        const bool hs_coo = mode_hess_coo(mode), hs_comp = mode_hess_comp(mode) && !grp.hc.empty();
+        const bool hs_coo = mode_hess_coo(mode);
+        const bool hs_comp = (mode_hess_comp(mode) || mode == M_HPROD) && !grp.hc.empty();
+        const bool jprod = mode == M_JPROD, jtprod = mode == M_JTPROD, hprod = mode == M_HPROD;
+        const bool graph_prod = mode_prod(mode) && prod;
         const bool want_struct = mode == M_STRUCT;
         // inputs staged in shared memory by the tile loop (s8 / s4: this thread's column of 8- and
         // 4-byte slots of the current buffer, slot j at [j * EXA_BLOCK])
@@ -1053,10 +1291,14 @@ struct Emitter {
             const bool obj = p.kind == EXA_OBJ;
             Want &w = want[pos];
             w.val = (mode == M_OBJ && obj) || (mode == M_CON && !obj) || all;
-            w.grad = (mode == M_GRAD && obj) || (mode == M_JAC && !obj) || all;
-            w.hess = mode_hess(mode) && p.nh() > 0;
-            w.row = !obj && (w.val || w.hess || want_struct);
+            w.grad = (mode == M_GRAD && obj) || ((mode == M_JAC || jprod || jtprod) && !obj) || all;
+            w.hess = (mode_hess(mode) || hprod) && p.nh() > 0;
+            w.row = !obj && (w.val || w.hess || want_struct || jprod || jtprod);
             const PatternGraph &G = PG[pos];
+            if (graph_prod) {  // J v: the row's product; J^T w, H v: below
+                if (jprod && prod->jv[pos] >= 0) roots.push_back(prod->jv[pos]);
+                continue;
+            }
             if (w.val) roots.push_back(G.value);
             if (w.grad) for (int s : p.jsym) roots.push_back(G.grad[s]);
             if (w.hess)
@@ -1066,6 +1308,9 @@ struct Emitter {
                     if (it != G.hess.end()) roots.push_back(it->second);
                 }
         }
+        if (graph_prod && !jprod)
+            for (int r : jtprod ? prod->jt : prod->hv)
+                if (r >= 0) roots.push_back(r);
         // inputs the roots need, by kind and precision
         std::set<int> syms, fields, params, fconsts;       // FP64 copies (loaded)
         std::set<int> fsyms, ffields, fparams, ffconsts;   // FP32 copies (converted)
@@ -1075,7 +1320,7 @@ struct Emitter {
                 if (seen[i]) return;
                 seen[i] = 1;
                 const SN &s = g.n[i];
-                if (s.op == S_IN) {
+                if (s.op == S_IN && s.ikind != 'V' && s.ikind != 'W') {
                     std::set<int> *d = s.ikind == 'X' ? &syms : s.ikind == 'D' ? &fields : s.ikind == 'P' ? &params : &fconsts;
                     std::set<int> *f = s.ikind == 'X' ? &fsyms : s.ikind == 'D' ? &ffields : s.ikind == 'P' ? &fparams : &ffconsts;
                     d->insert(s.iid);
@@ -1090,9 +1335,10 @@ struct Emitter {
         for (int pos : act) {
             const Pattern &p = pat(pos);
             if (want_struct) for (int s = 0; s < p.nsym; s++) idx_syms.insert(grp.sym[pos][s]);
+            if (jprod && want[pos].grad) for (int s = 0; s < p.nsym; s++) idx_syms.insert(grp.sym[pos][s]);
             if (want[pos].hess)
                 for (auto &pr : p.hpair)
-                    if (pr.first != pr.second) { idx_syms.insert(grp.sym[pos][pr.first]); idx_syms.insert(grp.sym[pos][pr.second]); }
+                    if (pr.first != pr.second || hprod) { idx_syms.insert(grp.sym[pos][pr.first]); idx_syms.insert(grp.sym[pos][pr.second]); }
         }
         // columns used as FP64 values (D) and as FP32 values (DF); in mixed mode f64 columns have an
         // FP32 copy (pm.f32) that FP32 uses load directly
@@ -1283,6 +1529,14 @@ struct Emitter {
                        << "    so.hcol[pm.hbase[" << P << "] + kk * " << p.nh() << " + " << j << "] = (int)(ga > gb ? gb : ga); }\n";
                 }
             }
+            for (size_t q = 0; q < grp.tsym.size(); q++)
+                os << "  so.tvar[pm.tbase + " << q << " * pm.n_inst + kk] = (int)(pm.xoff + i" << grp.tsym[q] << ");\n";
+            if (!grp.usym.empty()) {
+                os << "  if (so.uvar) {\n";
+                for (size_t q = 0; q < grp.usym.size(); q++)
+                    os << "    so.uvar[pm.ubase + " << q << " * pm.n_inst + kk] = (int)(pm.xoff + i" << grp.usym[q] << ");\n";
+                os << "  }\n";
+            }
             const int nhc = (int)grp.hc.size();
             if (nhc > 0) {
                 os << "  if (so.hcrow) {\n";
@@ -1299,12 +1553,28 @@ struct Emitter {
         if (!lazy)
             for (int s : syms)
                 os << "  const double X" << s << " = " << ld("X" + std::to_string(s), "x + pm.xoff + i" + std::to_string(s)) << ";\n";
+        // Products: the vector at the group's symbols (J v, H v) or at the rows (J^T w)
+        if (jprod || hprod) {
+            std::set<int> vs;
+            for (int pos : act)
+                if (jprod) vs.insert(grp.sym[pos].begin(), grp.sym[pos].end());
+            if (hprod) vs.insert(grp.usym.begin(), grp.usym.end());
+            // (the weights of H v and J^T w are named W, by pattern position)
+            for (int s : vs) os << "  const double V" << s << " = o.v[pm.xoff + i" << s << "];\n";
+        }
+        if (jtprod)
+            for (int pos : act) os << "  const double W" << pos << " = o.v[row" << pos << "];\n";
+        std::vector<char> started(grp.sym_root.size(), 0);  // J^T w, H v: sums begun per group symbol
+        auto accumulate = [&](int s, const std::string &term) {
+            os << (started[s] ? "  a" : "  double a") << s << (started[s] ? " += " : " = ") << term << ";\n";
+            started[s] = 1;
+        };
         // Pairs of different symbols whose slot doubles when both resolve to one variable: their
         // equality tests are taken once here, into one bit mask, so that the 64-bit indices are
         // dead once the gathers are issued instead of staying live until the Hessian.
         std::map<std::pair<int, int>, int> eqbit;
         for (int pos : act)
-            if (want[pos].hess)
+            if (want[pos].hess && !hprod)
                 for (auto &pr : pat(pos).hpair)
                     if (pr.first != pr.second) {
                         int ga = grp.sym[pos][pr.first], gb = grp.sym[pos][pr.second];
@@ -1435,7 +1705,7 @@ struct Emitter {
         // variable (2 a + 2 b = 2 (a + b) exactly).
         std::vector<int> hc_dup(grp.hc.size(), -1), hc_dsign(grp.hc.size(), 1);
         std::vector<std::vector<char>> hc_twice(grp.hc.size());  // per term of hc[c]: always doubled
-        if (hs_comp) {
+        if (hs_comp && !graph_prod) {
             std::map<std::vector<long long>, std::pair<int, int>> seen;  // normalised terms -> (sum, sign)
             for (size_t c = 0; c < grp.hc.size(); c++) {
                 std::vector<long long> key;
@@ -1479,6 +1749,21 @@ struct Emitter {
                 ready_pattern(pos);
                 if (j + 2 <= act.size() && j + 1 < act.size()) issue_pattern(act[j + 1]);
             }
+            if (graph_prod) {
+                if (hprod) os << "  const double W" << P << " = " << (obj ? "sigma" : "Y" + P) << ";\n";
+                if (!jprod) continue;
+                // a slot whose derivative is identically zero still multiplies its variable's value
+                std::string sum = "0.0";
+                if (prod->jv[pos] >= 0) {
+                    body({prod->jv[pos]}, name, &roots);
+                    sum = name.at(prod->jv[pos]);
+                }
+                for (int sy : p.jsym)
+                    if (g.zero(G.grad[sy])) sum += " + 0.0 * V" + std::to_string(grp.sym[pos][sy]);
+                if (p.kind == EXA_CON) os << "  if (act) o.c[row" << P << "] = " << sum << ";\n";
+                else os << "  if (act) o.abuf[pm.abase[" << P << "] + kk] = " << sum << ";\n";
+                continue;
+            }
             if (opt.by_pattern) {  // this pattern's arithmetic, right before its outputs
                 std::vector<int> mine;
                 if (w.val) mine.push_back(G.value);
@@ -1494,7 +1779,17 @@ struct Emitter {
             }
             // a block of S slots per instance: stage the warp's 32 x S values, then write the warp's
             // contiguous run of nact x S values with consecutive lanes on consecutive addresses
-            if (w.grad && p.nj() > 0) {
+            if (jprod) {
+                // the row's product: its derivatives are never stored
+                std::string sum;
+                for (int sy : p.jsym)
+                    sum += (sum.empty() ? "" : " + ") + widen(G.grad[sy]) + " * V" + std::to_string(grp.sym[pos][sy]);
+                if (sum.empty()) sum = "0.0";
+                if (p.kind == EXA_CON) os << "  if (act) o.c[row" << P << "] = " << sum << ";\n";
+                else os << "  if (act) o.abuf[pm.abase[" << P << "] + kk] = " << sum << ";\n";
+            } else if (jtprod) {
+                for (int sy : p.jsym) accumulate(grp.sym[pos][sy], widen(G.grad[sy]) + " * W" + P);
+            } else if (w.grad && p.nj() > 0) {
                 std::vector<std::string> vals;
                 for (int j = 0; j < p.nj(); j++) vals.push_back(widen(G.grad[p.jsym[j]]));
                 if (obj) staged("o.gbuf", "pm.gbase[" + P + "]", p.nj(), vals, nullptr, nullptr);
@@ -1532,7 +1827,7 @@ struct Emitter {
                     }
                     os << "  double " << hv << " = " << v << ";\n";
                     vals.push_back(hv);
-                    if (a != b) {
+                    if (a != b && !hprod) {
                         const int ga = grp.sym[pos][a], gb = grp.sym[pos][b];
                         const std::string c =
                             use_eqm ? "((eqm >> " + std::to_string(eqbit.at({std::min(ga, gb), std::max(ga, gb)})) + ") & 1ull)"
@@ -1565,19 +1860,34 @@ struct Emitter {
                 if (hs_coo) staged("o.hess", "pm.hbase[" + P + "]", p.nh(), vals, "o.hcsc", "o.hmap");
             }
         }
-        if (hs_comp) {  // per-instance FP64 sums of the Hessian slots that share (row, col) in the group
+        if (graph_prod && !jprod) {
+            const std::vector<int> &ss = jtprod ? grp.tsym : grp.usym, &rs = jtprod ? prod->jt : prod->hv;
+            body(roots, name);
+            for (size_t q = 0; q < ss.size(); q++)
+                if (rs[q] >= 0) accumulate(ss[q], name.at(rs[q]));
+        } else if (hs_comp) {  // per-instance FP64 sums of the Hessian slots that share (row, col) in the group
             for (size_t c = 0; c < grp.hc.size(); c++)
                 if (hc_dup[c] >= 0 && hc_started[hc_dup[c]]) {
                     const std::string src = "hc" + std::to_string(hc_dup[c]);
                     os << "  double hc" << c << " = " << (hc_dsign[c] < 0 ? "exa_neg(" + src + ")" : src) << ";\n";
                     hc_started[c] = 1;
                 }
+            // H v: an entry over two symbols contributes to both, so that two symbols that resolve to one
+            // variable need no doubling
+            if (hprod)
+                for (size_t c = 0; c < grp.hc.size(); c++) {
+                    if (!hc_started[c]) continue;
+                    const int ga = grp.hc_sym[c].first, gb = grp.hc_sym[c].second;
+                    const std::string h = "hc" + std::to_string(c);
+                    accumulate(ga, h + " * V" + std::to_string(gb));
+                    if (ga != gb) accumulate(gb, h + " * V" + std::to_string(ga));
+                }
             // sums over two different symbols that resolve to one variable: doubled as a whole
             std::string any;
             std::vector<std::pair<size_t, std::string>> dbl;
             for (size_t c = 0; c < grp.hc.size(); c++) {
                 const int ga = grp.hc_sym[c].first, gb = grp.hc_sym[c].second;
-                if (!hc_started[c] || ga == gb) continue;
+                if (!hc_started[c] || ga == gb || hprod) continue;
                 auto eb = eqbit.find({std::min(ga, gb), std::max(ga, gb)});
                 const std::string cond = use_eqm && eb != eqbit.end()
                                              ? "((eqm >> " + std::to_string(eb->second) + ") & 1ull)"
@@ -1591,8 +1901,20 @@ struct Emitter {
                 os << "  }\n";
             }
             std::vector<std::string> sums;
-            for (size_t c = 0; c < grp.hc.size(); c++) sums.push_back(hc_started[c] ? "hc" + std::to_string(c) : "0.0");
-            staged("o.hcomp", "pm.hcbase", (int)grp.hc.size(), sums, nullptr, nullptr);
+            if (!hprod)
+              for (size_t c = 0; c < grp.hc.size(); c++) sums.push_back(hc_started[c] ? "hc" + std::to_string(c) : "0.0");
+            if (!hprod) staged("o.hcomp", "pm.hcbase", (int)grp.hc.size(), sums, nullptr, nullptr);
+        }
+        // one array per group symbol: consecutive lanes store to consecutive addresses as they are, and
+        // the sums by variable read consecutive values where variables follow the instances
+        if (jtprod || hprod) {
+            const std::vector<int> &ss = jtprod ? grp.tsym : grp.usym;
+            const char *base = jtprod ? "pm.tbase" : "pm.ubase";
+            os << "  if (act) {\n";
+            for (size_t q = 0; q < ss.size(); q++)
+                os << "    o.prod[" << base << " + " << q << " * pm.n_inst + kk] = "
+                   << (started[ss[q]] ? "a" + std::to_string(ss[q]) : "0.0") << ";\n";
+            os << "  }\n";
         }
         os << "}\n";
         return os.str();
@@ -1681,6 +2003,16 @@ static const char *kFp64Helpers =
 #include "exa_fp64_sincos.inc"
     ;
 
+// The product kernels' sin and cos: a warp whose arguments are all below pi/4 in magnitude (usual for the
+// angle differences of a network) skips the reduction, 5 of the 20 FP64 operations; the quadrant is
+// then zero and r the argument itself, so the results are the same.
+static const char *kWarpSincos = R"(
+static __device__ __forceinline__ void exa_sincos64_warp(const double a, double* s, double* c) {
+  if (__all_sync(0xffffffffu, (__double2hiint(a) & 0x7fffffff) < 0x3fe921fb)) exa_sincos_poly(a, 0, s, c);
+  else exa_sincos64(a, s, c);
+}
+)";
+
 // Reductions of the fused step (ExaRed), run by one CTA over [p0, p1).  Values written by other
 // CTAs during the kernel (COO slots, compressed sums, gradient and augmentation buffers,
 // constraint base values) are read through L2 (ld.global.cg); the index arrays are constant.
@@ -1755,6 +2087,14 @@ static __device__ void exa_step_task(const ExaStep& st, const ExaTask& tk, int* 
 std::string generate_source(const std::vector<Pattern> &pats, const std::vector<Group> &groups,
                             const CodegenOptions &opt_in, std::string *err, int *dsmem) {
     CodegenOptions opt = opt_in;
+    if (opt.products) {
+        CodegenOptions plain;
+        plain.precision = opt.precision;
+        plain.block = opt.block;
+        plain.bounds_check = opt.bounds_check;
+        plain.products = true;
+        opt = plain;
+    }
     if (opt.lanes > 1) opt.prefetch = 0;  // one or the other
     if (opt.fused_step) {  // the fused step kernels take plain tiles
         opt.stage = 0;
@@ -1767,7 +2107,8 @@ std::string generate_source(const std::vector<Pattern> &pats, const std::vector<
         if (opt.bounds_check) opt.stage = 0;
     }
     if (dsmem)
-        for (int m = 0; m < M_COUNT; m++) dsmem[m] = 0;
+        for (int m = 0; m < M_COUNT; m++)
+            if (mode_prod(m) == opt.products) dsmem[m] = 0;
     std::ostringstream src;
     const bool mixed = opt.precision == EXA_MIXED_FP32;
     src << "// generated by exa_lower.cpp (" << (mixed ? "mixed FP32/FP64" : "FP64") << ")\n";
@@ -1780,6 +2121,7 @@ std::string generate_source(const std::vector<Pattern> &pats, const std::vector<
     if (mixed) src << kMixedHelpers;
     src << kExactHelpers;
     src << kFp64Helpers;
+    if (opt.products) src << kWarpSincos;
     if (opt.fused_step) src << kStepHelpers;
     if (opt.stage)
         src << "// cp.async of one 8- or 4-byte input into a shared-memory slot (both addresses aligned to\n"
@@ -1806,7 +2148,23 @@ std::string generate_source(const std::vector<Pattern> &pats, const std::vector<
             }
         }
     }
+    std::vector<ProdGraph> prods;
+    if (opt.products) {
+        // Resident CTAs of 64 threads that the product kernels are held to: 16 (64 registers) for plain
+        // arithmetic and sin/cos, 12 (80) where divisions and library functions would spill.  Measured, us
+        // for J v, J^T w and H v together, uncapped / 12 / 16: 30,000-bus network 63.0 / 66.3 / 54.9, 32
+        // networks 153.8 / 150.6 / 152.6, 100,000-step rocket (exp, divisions) 135 / 127 / 140.
+        bool plain = true;
+        for (const Graph &gr : graphs)
+            for (const SN &n : gr.n) plain = plain && (n.op <= S_MUL || n.op == S_SIN || n.op == S_COS || n.op == S_CVT ||
+                                                      n.op == S_SINR || n.op == S_COSR);
+        src << "#undef EXA_BOUNDS\n#define EXA_BOUNDS __launch_bounds__(EXA_BLOCK, " << (plain ? 16 : 12) << ")\n";
+    }
+    if (opt.products && !mixed)
+        for (size_t gi = 0; gi < groups.size(); gi++)
+            prods.push_back(build_products(pats, groups[gi], graphs[gi], pgs[gi]));
     for (int m = 0; m < M_COUNT; m++) {
+        if (mode_prod(m) != opt.products) continue;
         std::vector<int> gl;
         std::map<int, int> nsets;  // group -> warp sets (> 1 only when split)
         int S8 = 0, S4 = 0;        // staged slots per thread (largest over the kernel's groups)
@@ -1825,6 +2183,7 @@ std::string generate_source(const std::vector<Pattern> &pats, const std::vector<
             gl.push_back((int)gi);
             Emitter e(pats, groups[gi], graphs[gi], pgs[gi], opt);
             e.st_budget = st_budget;
+            if (!prods.empty()) e.prod = &prods[gi];
             const std::vector<std::vector<int>> sets = group_sets(pats, groups[gi], (Mode)m, opt.lanes);
             if (sets.size() == 1) {
                 src << e.function((int)gi, (Mode)m, sets[0]);
@@ -1872,7 +2231,9 @@ std::string generate_source(const std::vector<Pattern> &pats, const std::vector<
             src << "  asm volatile(\"griddepcontrol.launch_dependents;\" ::: \"memory\");\n"
                    "  asm volatile(\"griddepcontrol.wait;\" : \"+l\"(x), \"+l\"(y), \"+l\"(th) : : \"memory\");\n";
         if (objred) src << "  __shared__ double red[EXA_BLOCK / 32];\n";
-        if (m != M_STRUCT)
+        if (mode_prod(m))
+            src << "  double* ws = nullptr;\n";
+        else if (m != M_STRUCT)
             src << "  __shared__ double stage[EXA_BLOCK * " << smax << "];\n"
                    "  double* __restrict__ ws = stage + (threadIdx.x & ~31u) * " << smax << ";\n";
         else

@@ -42,18 +42,26 @@ def test_segment_lengths(spread, batch):
     out = m.eval_all(x, y, 1.0, csc=True)
     got = {k: t.cpu().numpy() for k, t in out.items()}
     one = dict(f=m.obj(x), g=m.grad(x), c=m.cons(x), jac_csc=m.jac_csc(x), hess_csc=m.hess_csc(x, y))
+    vs = [rng.uniform(0.5, 1.5, f.nvar) for f in flats]
+    ws = [rng.uniform(0.5, 1.5, f.ncon) for f in flats]
+    v, w = (torch.as_tensor(np.concatenate(a), device="cuda") for a in (vs, ws))
+    one.update(jv=m.jprod(x, v), jtw=m.jtprod(x, w), hv=m.hprod(x, y, 1.0, v))
     one = {k: t.cpu().numpy() for k, t in one.items()}
     orc = [oracle.Oracle(f) for f in flats]
     ref = dict(f=np.array([sum(o.obj(a) for o, a in zip(orc, xs))]),
                g=np.concatenate([o.grad(a) for o, a in zip(orc, xs)]),
                c=np.concatenate([o.cons(a) for o, a in zip(orc, xs)]),
                jac_csc=np.concatenate([o.jac_csc(a) for o, a in zip(orc, xs)]),
-               hess_csc=np.concatenate([o.hess_csc(a, b, 1.0) for o, a, b in zip(orc, xs, ys)]))
+               hess_csc=np.concatenate([o.hess_csc(a, b, 1.0) for o, a, b in zip(orc, xs, ys)]),
+               jv=np.concatenate([o.jprod(a, b) for o, a, b in zip(orc, xs, vs)]),
+               jtw=np.concatenate([o.jtprod(a, b) for o, a, b in zip(orc, xs, ws)]),
+               hv=np.concatenate([o.hprod(a, b, 1.0, c) for o, a, b, c in zip(orc, xs, ys, vs)]))
     # every term is positive: two orders of a sum of n terms differ by at most 2 (n + 4) ulp of the sum
-    # (four operations form a term), and the objective adds all of them
+    # (at most four operations form a term; a variable's second-order sum has the terms of the objective
+    # and of the rows), and the objective adds all of them
     n = max(sum(v) for v in lists)
     for k, r in ref.items():
-        tol = 2 * ((len(lists) * n if k == "f" else max(max(v) for v in lists)) + 4) * 2.0 ** -53
-        for a in (got[k], one[k]):
+        tol = 2 * ((len(lists) * n if k == "f" else 2 * max(max(v) for v in lists)) + 4) * 2.0 ** -53
+        for a in [d[k] for d in (got, one) if k in d]:
             assert a.shape == r.shape
             assert np.all(np.abs(a - r) <= tol * np.abs(r)), k

@@ -6,7 +6,8 @@
 // and on models that fit the L2 cache it takes a few microseconds, less than the gap between two
 // dependent launches.  So all jobs of a step are blocks of one kernel, and that kernel is launched
 // with programmatic stream serialization: its blocks become resident while the evaluation kernel
-// drains, load their indices (constant since creation) and only then wait for its results.
+// drains (when its blocks have finished their tiles), load their indices (constant since creation) and
+// only then wait for its results.
 //
 // Measured (GB300, whole exa_eval_all steps; before: one kernel per reduction on three streams, the
 // multi-entry CSC segments added onto a first pass): 1000-variable model 25.4 -> 15.4 us, 30,000-bus
@@ -23,12 +24,11 @@ namespace exa_red {
 
 // Waits until the kernels this one depends on have completed and their writes are visible (no-op
 // for an ordinary launch), and returns src: loads through the returned pointer cannot be moved ahead of
-// the wait, whatever kind of load they are.  allow_next lets the next kernel's blocks be scheduled.
+// the wait, whatever kind of load they are.
 static __device__ __forceinline__ const double *wait_inputs(const double *src) {
     asm volatile("griddepcontrol.wait;" : "+l"(src) : : "memory");
     return src;
 }
-static __device__ __forceinline__ void allow_next() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
 
 enum Kind {
     PERM = 0,  // dst[p] = src[perm[p]] for perm[p] >= 0; 0.0 for EMPTY; nothing for ELSEWHERE
@@ -174,7 +174,6 @@ static __device__ __forceinline__ double block_sum(double s, double *buf) {
 
 static __global__ void __launch_bounds__(THREADS, 6) k_reduce(const __grid_constant__ Jobs J) {
     __shared__ double buf[(THREADS / 32) * PIECE];
-    allow_next();
     // block of the job list: as launched, or every `every`-th one a block of a sum
     int vb = (int)blockIdx.x;
     if (J.every > 1) {
@@ -237,7 +236,6 @@ static __global__ void __launch_bounds__(THREADS, 6) k_reduce(const __grid_const
 // f[0] = the sum of n objective partials, one CTA (the whole launch of the objective callbacks).
 static __global__ void __launch_bounds__(1024) k_obj_final(const double *part, int n, double *f) {
     __shared__ double buf[32];
-    allow_next();
     part = wait_inputs(part);
     const double t = block_sum(strided_sum(part, nullptr, 0, n, threadIdx.x, blockDim.x), buf);
     if (threadIdx.x == 0) f[0] = t;

@@ -189,13 +189,14 @@ struct SegList {
 // A gather-sum over a sorted permutation, split by segment length into independent jobs (exa_reduce.h)
 // when it is built: elements with one entry or none are a plain gather over the codes `first`
 // (most CSC entries have one contributor, so most of the work is a permutation); short segments are
-// added up in ascending order by one lane, segments above SHORT_MAX entries by a warp, and above
-// WARP_MAX by blocks of CHUNK_LEN entries whose partial sums a second launch adds up.  CSC sums are
+// added up in ascending order by one lane, segments above SHORT_MAX entries by a warp, above WARP_MAX by
+// a block, and above BLOCK_MAX by blocks of CHUNK_LEN entries whose partial sums a second launch adds
+// up.  CSC sums are
 // `ordered`: every duplicate sum is short, i.e. in ascending COO order.
 struct GatherSum {
     int n = 0;              // positions of `first` (0: every element is in a list)
     int *first = nullptr;
-    SegList sh, md, lg;
+    SegList sh, md, bl, lg;
     int *cptr = nullptr;    // pieces of the long segments: the entries [cptr[2 c], cptr[2 c + 1])
     int *lcptr = nullptr;   // lcptr[i] = first piece of long segment i (n + 1)
     std::vector<int> h_lcptr;
@@ -254,18 +255,19 @@ struct exa_model {
         std::array<const void *, 10> key;
         cudaGraphExec_t exec;
         uint64_t last_use;
+        bool stamped;
     };
     std::vector<GraphEntry> graphs;
     uint64_t graph_clock = 0;
     int graph_kernels = 0;  // kernel launches in the most recently captured exa_eval_all graph
     bool use_graphs = true;
     cudaStream_t cap_stream = nullptr;
-    // side streams of exa_eval_all, forked from and joined back into the model stream: 0 the split
-    // mode's first-order reductions (and member chunks' reductions), 1 the timing event of the graph
-    cudaStream_t side[4] = {};
+    // side stream of exa_eval_all, forked from and joined back into the model stream: the split mode's
+    // first-order reductions, and member chunks' reductions
+    cudaStream_t side = nullptr;
     // device buffers of exa_eval_all_host: x, y, f, g, c, jac, hess, jac_csc, hess_csc
     double *d_host_io[9] = {};
-    cudaEvent_t ev_fork = nullptr, ev_first = nullptr, ev_join[4] = {};
+    cudaEvent_t ev_first = nullptr, ev_join = nullptr;
     double *d_theta = nullptr;
     int *d_status = nullptr;
     int *d_jrow = nullptr, *d_jcol = nullptr, *d_hrow = nullptr, *d_hcol = nullptr, *d_gvar = nullptr, *d_arow = nullptr;
@@ -308,6 +310,9 @@ struct exa_model {
     // the cached graphs too); exa_stat "eval_kernel_ms" reads them
     cudaEvent_t ev_k0 = nullptr, ev_k1 = nullptr;
     bool ev_k_valid = false;
+    // ... or two device timer stamps, in graphs of one evaluation kernel and its reductions
+    unsigned long long *d_stamp = nullptr;
+    bool stamped = false;  // the latest call used the stamps
     bool grad_compact = false;
     int n_gseg = 0;
     int *d_gsegptr = nullptr, *d_gsegvar = nullptr;
@@ -368,16 +373,12 @@ void free_all(exa_model *m) {
     m->graphs.clear();
     if (m->cap_stream) cudaStreamDestroy(m->cap_stream);
     m->cap_stream = nullptr;
-    for (int s = 0; s < 4; s++) {
-        if (m->side[s]) cudaStreamDestroy(m->side[s]);
-        if (m->ev_join[s]) cudaEventDestroy(m->ev_join[s]);
-        m->side[s] = nullptr;
-        m->ev_join[s] = nullptr;
+    if (m->side) cudaStreamDestroy(m->side);
+    m->side = nullptr;
+    for (cudaEvent_t *e : {&m->ev_join, &m->ev_first}) {
+        if (*e) cudaEventDestroy(*e);
+        *e = nullptr;
     }
-    if (m->ev_fork) cudaEventDestroy(m->ev_fork);
-    if (m->ev_first) cudaEventDestroy(m->ev_first);
-    m->ev_fork = nullptr;
-    m->ev_first = nullptr;
     for (cudaEvent_t &e : m->ev_chunk) {
         if (e) cudaEventDestroy(e);
         e = nullptr;
@@ -444,6 +445,16 @@ exa_status nvrtc_compile(exa_model *m, const std::string &src, std::vector<char>
 // pattern trees and options (batch members, or the same model created twice) compile once.
 std::mutex g_cubin_mu;
 std::map<std::string, std::shared_ptr<std::vector<char>>> g_cubins;
+// The product kernels' source by the evaluation kernels' source (which holds the same patterns, groups,
+// precision and layout), so that a model whose modules are cached generates one source; cleared with
+// the modules.
+std::map<std::string, std::string> g_prod_src;
+
+void trim_cache() {  // with g_cubin_mu held
+    if (g_cubins.size() <= 64) return;
+    g_cubins.clear();
+    g_prod_src.clear();
+}
 
 // Compiles the kernels of several code-generator variants into the module cache at once, one
 // thread per variant (NVRTC is thread-safe): the tuner then loads each variant from the cache.
@@ -464,7 +475,7 @@ void precompile(const exa_model *m, const std::vector<exa::CodegenOptions> &vari
             auto cubin = std::make_shared<std::vector<char>>();
             if (nvrtc_compile(&scratch, src, *cubin) != EXA_OK) return;
             std::lock_guard<std::mutex> lk(g_cubin_mu);
-            if (g_cubins.size() > 64) g_cubins.clear();
+            trim_cache();
             g_cubins[src] = cubin;
         });
     for (std::thread &t : th) t.join();
@@ -483,7 +494,7 @@ exa_status cubin_of(exa_model *m, const std::string &src, std::shared_ptr<std::v
     auto cubin = std::make_shared<std::vector<char>>();
     if (exa_status e = nvrtc_compile(m, src, *cubin)) return e;
     std::lock_guard<std::mutex> lk(g_cubin_mu);
-    if (g_cubins.size() > 64) g_cubins.clear();
+    trim_cache();
     g_cubins[src] = *out = cubin;
     return EXA_OK;
 }
@@ -635,6 +646,7 @@ class Reduction {
             k.n = gs.h_lcptr[s1] - c0;
             k.ptr = gs.cptr + 2 * (i64)c0;
             k.perm = gs.lg.perm;
+            k.add = 0;
             k.dst = gs.part + c0;
             push(J, k);
             k = j;
@@ -645,6 +657,7 @@ class Reduction {
             k.src = gs.part;
             push(J2, k);
         }
+        list(gs.bl, exa_red::BSEG);
         list(gs.md, exa_red::WSEG);
         list(gs.sh, exa_red::SEG);
         if (gs.n > 0) {
@@ -675,6 +688,8 @@ class Reduction {
         else zero = f;
     }
     double *zero = nullptr;  // an objective without partials
+    bool empty() const { return !J.nj; }
+    void stamp(unsigned long long *t) { J.stamp = t; }
 
     exa_status launch(exa_model *m, cudaStream_t st, bool overlap) {
         if (zero) CR(cudaMemsetAsync(zero, 0, sizeof(double), st));
@@ -684,7 +699,7 @@ class Reduction {
             // long dependent chains first, streaming jobs last
             std::stable_sort(js->j, js->j + js->nj, [](const exa_red::Job &a, const exa_red::Job &b) {
                 auto rank = [](const exa_red::Job &j) {
-                    return j.kind == exa_red::OBJ ? 0 : j.kind == exa_red::CHUNK ? 1 : j.kind == exa_red::WSEG ? 2
+                    return j.kind == exa_red::OBJ ? 0 : j.kind == exa_red::CHUNK || j.kind == exa_red::BSEG ? 1 : j.kind == exa_red::WSEG ? 2
                            : j.kind == exa_red::SEG ? 3 : j.kind == exa_red::PERM ? 4 : 5;
                 };
                 return rank(a) < rank(b);
@@ -699,7 +714,7 @@ class Reduction {
                 case exa_red::PERM: j.wide = j.n >= wide * 2048; blocks += (j.n + (j.wide ? 2047 : 511)) / (j.wide ? 2048 : 512); break;
                 case exa_red::SEG: j.wide = j.n >= wide * 512; blocks += (j.n + (j.wide ? 511 : 255)) / (j.wide ? 512 : 256); break;
                 case exa_red::WSEG: case exa_red::CSUM: blocks += (j.n + 7) / 8; break;
-                case exa_red::CHUNK: blocks += j.n; break;
+                case exa_red::CHUNK: case exa_red::BSEG: blocks += j.n; break;
                 case exa_red::OBJ: blocks += 1; break;
                 default: blocks += ((i64)(j.n + 31) / 32 - j.lo / 32 + 255) / 256; break;
                 }
@@ -855,7 +870,11 @@ exa_status build_gather_sum(exa_model *m, Scratch &S, const int *ptr, const int 
     }
     if (exa_status e = build_seg_list(m, S, ptr, perm, rows, n, lo, exa_red::SHORT_MAX, true, &gs->sh)) return e;
     if (exa_status e = build_seg_list(m, S, ptr, perm, rows, n, exa_red::SHORT_MAX, exa_red::WARP_MAX, false, &gs->md)) return e;
-    if (exa_status e = build_seg_list(m, S, ptr, perm, rows, n, exa_red::WARP_MAX, INT32_MAX, false, &gs->lg)) return e;
+    if (longest > exa_red::WARP_MAX)
+        if (exa_status e = build_seg_list(m, S, ptr, perm, rows, n, exa_red::WARP_MAX, exa_red::BLOCK_MAX, false, &gs->bl))
+            return e;
+    if (longest > exa_red::BLOCK_MAX)
+        if (exa_status e = build_seg_list(m, S, ptr, perm, rows, n, exa_red::BLOCK_MAX, INT32_MAX, false, &gs->lg)) return e;
     if (!gs->lg.n) return EXA_OK;
     std::vector<int> range(2 * (size_t)gs->lg.n), piece;
     CR(cudaMemcpy(range.data(), gs->lg.ptr, sizeof(int) * range.size(), cudaMemcpyDeviceToHost));
@@ -909,7 +928,7 @@ exa_status build_member_bounds(exa_model *m) {
     // element at or above the member's first
     auto lists = [&](GatherSum &gs, const std::vector<long long> &keys) -> exa_status {
         for (long long v : keys) gs.mb.push_back((int)v);
-        for (SegList *L : {&gs.sh, &gs.md, &gs.lg})
+        for (SegList *L : {&gs.sh, &gs.md, &gs.bl, &gs.lg})
             if (L->n)
                 if (exa_status e = lower(L->row, L->n, keys, L->mb)) return e;
         return EXA_OK;
@@ -1166,10 +1185,20 @@ exa_status setup_kernels(exa_model *m, int block, int min_blocks = 0) {
     if (!gerr.empty()) return fail(m, EXA_E_INTERNAL, gerr);
     std::string psrc;  // the product kernels, once per model
     if (!m->lib_prod) {
-        cg.block = PROD_BLOCK;
-        cg.products = true;
-        psrc = exa::generate_source(m->pats, m->groups, cg, &gerr, m->dsmem);
-        if (!gerr.empty()) return fail(m, EXA_E_INTERNAL, gerr);
+        {
+            std::lock_guard<std::mutex> lk(g_cubin_mu);
+            auto it = g_prod_src.find(src);
+            if (it != g_prod_src.end()) psrc = it->second;
+        }
+        if (psrc.empty()) {
+            cg.block = PROD_BLOCK;
+            cg.products = true;
+            psrc = exa::generate_source(m->pats, m->groups, cg, &gerr);
+            if (!gerr.empty()) return fail(m, EXA_E_INTERNAL, gerr);
+            std::lock_guard<std::mutex> lk(g_cubin_mu);
+            if (g_prod_src.size() >= 64) g_prod_src.clear();
+            g_prod_src[src] = psrc;
+        }
     }
     dump_source(src + psrc);
     if (m->lib) {
@@ -1834,6 +1863,7 @@ exa_status create_impl(const exa_model_desc *const *descs, int nb, const exa_opt
     CR(dalloc(m, &m->d_theta, m->npar));
     CR(dalloc(m, &m->d_status, 1));
     CR(cudaMemset(m->d_status, 0, sizeof(int)));
+    CR(dalloc(m, &m->d_stamp, 2));
     std::vector<ExaPM> pms((size_t)nb * ng);
     for (int b = 0; b < nb; b++) {
         const exa_model_desc &d = *descs[b];
@@ -2278,6 +2308,7 @@ static exa_status record_eval_event(exa_model *m, cudaEvent_t *ev, cudaStream_t 
     CR(cudaStreamIsCapturing(m->stream, &cs));
     const bool own_capture = cs != cudaStreamCaptureStatusNone && m->stream == m->cap_stream;
     if (cs != cudaStreamCaptureStatusNone && !own_capture) return EXA_OK;
+    m->stamped = false;
     if (!*ev) CR(cudaEventCreate(ev));
     if (own_capture) CR(cudaEventRecordWithFlags(*ev, st, cudaEventRecordExternal));
     else CR(cudaEventRecord(*ev, st));
@@ -2286,7 +2317,7 @@ static exa_status record_eval_event(exa_model *m, cudaEvent_t *ev, cudaStream_t 
 }
 
 // exa_eval_all over member chunks: for every chunk, its evaluation kernel(s) on the model stream,
-// then, on side stream 0 once that chunk's kernel has finished, its Jacobian CSC, Hessian CSC,
+// then, on the side stream once that chunk's kernel has finished, its Jacobian CSC, Hessian CSC,
 // gradient and constraint reductions over the chunk's own ranges of every output (members own
 // contiguous ranges of variables, rows, tiles and CSC positions).  The evaluation of the next chunk
 // overlaps these reductions.  The objective sum follows the last evaluation; the host copies of
@@ -2294,14 +2325,11 @@ static exa_status record_eval_event(exa_model *m, cudaEvent_t *ev, cudaStream_t 
 static exa_status eval_all_chunked(exa_model *m, const double *x, const double *y, double sigma, double *f, double *g,
                                    double *c, double *jac_csc, double *hess_csc, ExaOut o,
                                    Mode mode, Mode hmode, bool split, bool jdirect, bool hdirect, bool hcomp) {
-    if (!m->ev_fork) CR(cudaEventCreateWithFlags(&m->ev_fork, cudaEventDisableTiming));
-    for (int s = 0; s < 3; s++) {
-        if (!m->side[s]) CR(side_stream(&m->side[s]));
-        if (!m->ev_join[s]) CR(cudaEventCreateWithFlags(&m->ev_join[s], cudaEventDisableTiming));
-    }
+    if (!m->side) CR(side_stream(&m->side));
+    if (!m->ev_join) CR(cudaEventCreateWithFlags(&m->ev_join, cudaEventDisableTiming));
     for (int k = 0; k < m->nchunks; k++)
         if (!m->ev_chunk[k]) CR(cudaEventCreateWithFlags(&m->ev_chunk[k], cudaEventDisableTiming));
-    cudaStream_t ps = m->side[0];
+    cudaStream_t ps = m->side;
     const bool jside = jac_csc && !jdirect && m->nnzj_csc;
     const bool hside = (hcomp || (hess_csc && !hdirect)) && m->nnzh_csc;
     ExaOut o1 = o, o2{};
@@ -2345,8 +2373,8 @@ static exa_status eval_all_chunked(exa_model *m, const double *x, const double *
     }
     if (f)
         if (exa_status e = obj_final(m, m->d_objpart, nparts, f, m->stream, false)) return e;
-    CR(cudaEventRecord(m->ev_join[0], ps));
-    CR(cudaStreamWaitEvent(m->stream, m->ev_join[0], 0));
+    CR(cudaEventRecord(m->ev_join, ps));
+    CR(cudaStreamWaitEvent(m->stream, m->ev_join, 0));
     return EXA_OK;
 }
 
@@ -2517,9 +2545,12 @@ static exa_status eval_all_launches(exa_model *m, const double *x, const double 
         return eval_all_chunked(m, x, y, sigma, f, g, c, jac_csc, hess_csc, o, want_h ? mode : exa::M_FIRST,
                                 hmode, want_h && m->split_all, jdirect, hdirect, hcomp);
     // The evaluation kernel(s), then every reduction as jobs of one launch.  In split mode the
-    // first-order reductions run on side stream 0 as soon as the first-order kernel has, overlapping
+    // first-order reductions run on the side stream as soon as the first-order kernel has, overlapping
     // the second-order kernel (the reductions move bytes, the second-order kernel keeps the FP64 pipe
-    // busy), and only the Hessian CSC follows the second.
+    // busy), and only the Hessian CSC follows the second.  The captured graph of one evaluation kernel and
+    // its reductions holds just these two nodes, joined by a programmatic edge: the kernels stamp the
+    // device time themselves, because two event-record nodes took 4 us of each step (1000-variable
+    // model 15.0 -> 11.1 us, 500-bus network 19.1 -> 15.2 us).
     const bool split = want_h && m->split_all;
     Reduction first, second;
     if (f) first.obj(m->d_objpart, eval_grid(m, split ? exa::M_FIRST : mode, m->ntiles[split ? exa::M_FIRST : mode]), f);
@@ -2532,15 +2563,19 @@ static exa_status eval_all_launches(exa_model *m, const double *x, const double 
     cudaStreamCaptureStatus cs = cudaStreamCaptureStatusNone;
     CR(cudaStreamIsCapturing(m->stream, &cs));
     const bool own_capture = cs != cudaStreamCaptureStatusNone && m->stream == m->cap_stream;
-    if (split || own_capture) {
-        for (cudaEvent_t *e : {&m->ev_fork, &m->ev_first})
-            if (!*e) CR(cudaEventCreateWithFlags(e, cudaEventDisableTiming));
-        for (int s = 0; s < 2; s++) {
-            if (!m->side[s]) CR(side_stream(&m->side[s]));
-            if (!m->ev_join[s]) CR(cudaEventCreateWithFlags(&m->ev_join[s], cudaEventDisableTiming));
-        }
+    if (split) {
+        if (!m->ev_first) CR(cudaEventCreateWithFlags(&m->ev_first, cudaEventDisableTiming));
+        if (!m->side) CR(side_stream(&m->side));
+        if (!m->ev_join) CR(cudaEventCreateWithFlags(&m->ev_join, cudaEventDisableTiming));
     }
-    if (exa_status e = record_eval_event(m, &m->ev_k0, m->stream)) return e;
+    const bool stamps = own_capture && !split && !first.empty();
+    if (stamps) {
+        m->stamped = true;
+        o.stamp = m->d_stamp;
+        first.stamp(m->d_stamp + 1);
+    } else if (exa_status e = record_eval_event(m, &m->ev_k0, m->stream)) {
+        return e;
+    }
     if (split) {  // first order and second order as two kernels
         ExaOut o1 = o, o2{};
         o1.hess = nullptr;
@@ -2556,25 +2591,15 @@ static exa_status eval_all_launches(exa_model *m, const double *x, const double 
     } else {
         if (exa_status e = launch_eval(m, mode, x, y, sigma, o)) return e;
     }
-    // The second timing event follows the evaluation kernel on a branch of its own in the captured
-    // graph, so that the reductions depend on that kernel directly (a programmatic edge); in plain
-    // launches it is recorded in stream order.
-    if (own_capture) {
-        CR(cudaEventRecord(m->ev_fork, m->stream));
-        CR(cudaStreamWaitEvent(m->side[1], m->ev_fork, 0));
-        if (exa_status e = record_eval_event(m, &m->ev_k1, m->side[1])) return e;
-        CR(cudaEventRecord(m->ev_join[1], m->side[1]));
-    } else if (exa_status e = record_eval_event(m, &m->ev_k1, m->stream)) {
-        return e;
-    }
+    if (!stamps)
+        if (exa_status e = record_eval_event(m, &m->ev_k1, m->stream)) return e;
     if (split) {
-        CR(cudaStreamWaitEvent(m->side[0], m->ev_first, 0));
-        if (exa_status e = first.launch(m, m->side[0], false)) return e;
-        CR(cudaEventRecord(m->ev_join[0], m->side[0]));
+        CR(cudaStreamWaitEvent(m->side, m->ev_first, 0));
+        if (exa_status e = first.launch(m, m->side, false)) return e;
+        CR(cudaEventRecord(m->ev_join, m->side));
     }
     if (exa_status e = hr.launch(m, m->stream, true)) return e;
-    if (split) CR(cudaStreamWaitEvent(m->stream, m->ev_join[0], 0));
-    if (own_capture) CR(cudaStreamWaitEvent(m->stream, m->ev_join[1], 0));
+    if (split) CR(cudaStreamWaitEvent(m->stream, m->ev_join, 0));
     return EXA_OK;
 }
 
@@ -2594,6 +2619,7 @@ static exa_status eval_all_cached(exa_model *m, const double *x, const double *y
     for (auto &ge : m->graphs)
         if (ge.key == key) {
             ge.last_use = ++m->graph_clock;
+            m->stamped = ge.stamped;
             CR(cudaGraphLaunch(ge.exec, m->stream));
             return EXA_OK;
         }
@@ -2634,7 +2660,7 @@ static exa_status eval_all_cached(exa_model *m, const double *x, const double *y
         cudaGraphExecDestroy(lru->exec);
         m->graphs.erase(lru);
     }
-    m->graphs.push_back({key, exec, ++m->graph_clock});
+    m->graphs.push_back({key, exec, ++m->graph_clock, m->stamped});
     CR(cudaGraphLaunch(exec, m->stream));
     return EXA_OK;
 }
@@ -2737,8 +2763,8 @@ exa_status exa_eval_all_host(exa_model *m, const double *x, const double *y, dou
         return EXA_OK;
     };
     m->post_chunk = [&](int k) -> exa_status {
-        // chunk k's reductions ran on side stream 0 after its evaluation kernel
-        CR(cudaEventRecord(m->ev_out[k], m->side[0]));
+        // chunk k's reductions ran on the side stream after its evaluation kernel
+        CR(cudaEventRecord(m->ev_out[k], m->side));
         CR(cudaStreamWaitEvent(m->d2h, m->ev_out[k], 0));
         for (int a = 3; a < 9; a++) {
             if (!staged[a]) continue;
@@ -2912,7 +2938,12 @@ exa_status exa_stat(const exa_model *m, const char *key, double *value) {
     else if (k == "eval_fused_step") *value = m->fused_step;
     else if (k == "eval_kernel_ms") {  // evaluation kernel(s) of the latest exa_eval_all step
         float ms = -1.0f;
-        if (!m->ev_k_valid || cudaEventSynchronize(m->ev_k1) != cudaSuccess ||
+        unsigned long long t[2];
+        if (m->stamped) {  // device timer (ns) around the kernel
+            if (cudaSetDevice(m->device) == cudaSuccess && cudaDeviceSynchronize() == cudaSuccess &&
+                cudaMemcpy(t, m->d_stamp, sizeof t, cudaMemcpyDeviceToHost) == cudaSuccess && t[1] >= t[0])
+                ms = (float)(1e-6 * (double)(t[1] - t[0]));
+        } else if (!m->ev_k_valid || cudaEventSynchronize(m->ev_k1) != cudaSuccess ||
             cudaEventElapsedTime(&ms, m->ev_k0, m->ev_k1) != cudaSuccess)
             ms = -1.0f;
         *value = ms;

@@ -54,6 +54,7 @@
         const int *hmap;          /* Hessian COO slot -> CSC position */                            \
         double *hcomp;            /* if set: per-instance sums of the group's equal Hessian pairs */\
         int *status;              /* device fault word (bounds) */                                  \
+        unsigned long long *stamp;/* if set: [0] = device time (ns) at which the kernel started */   \
         const double *v;          /* products: the vector */                                        \
         double *prod;             /* products: J^T w or H v terms per instance and group symbol */  \
     };                                                                                              \

@@ -2232,6 +2232,8 @@ std::string generate_source(const std::vector<Pattern> &pats, const std::vector<
         // overlap, 27 us this way; a 30,000-bus network's products 54, 59 and 42 us.)
         if (m != M_STRUCT)
             src << "  asm volatile(\"griddepcontrol.wait;\" : \"+l\"(x), \"+l\"(y), \"+l\"(th) : : \"memory\");\n";
+        if (mode_all(m) || m == M_FIRST)
+            src << "  if (o.stamp && blockIdx.x == 0 && threadIdx.x == 0) asm volatile(\"mov.u64 %0, %%globaltimer;\" : \"=l\"(*o.stamp) : : \"memory\");\n";
         if (objred) src << "  __shared__ double red[EXA_BLOCK / 32];\n";
         if (mode_prod(m))
             src << "  double* ws = nullptr;\n";

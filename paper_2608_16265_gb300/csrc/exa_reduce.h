@@ -35,6 +35,7 @@ enum Kind {
     SEG,       // dst[row[s]] = the values src[perm[q]], q in [ptr[s], ptr[s+1]), added in ascending q
     WSEG,      // the same over q in [ptr[2 s], ptr[2 s + 1]) for longer segments: one warp each, lanes'
                // strided sums, then a tree
+    BSEG,      // the same, one block each
     CHUNK,     // dst[c] = sum of src[perm[q]], q in [ptr[2 c], ptr[2 c + 1]) (a piece of a long segment)
     CSUM,      // dst[row[s]] = the pieces src[ptr[s] .. ptr[s+1]) of long segment s
     OBJ,       // dst[0] = sum of the objective partials src[0 .. n)
@@ -47,7 +48,7 @@ struct Job {
     int blk0 = 0;    // first block of the job
     int n = 0;       // positions, segments, pieces or partials
     int wide = 0;    // PERM: 8 positions per thread instead of 2; SEG: 64 segments per warp instead of 32
-    int add = 0;     // SEG, WSEG, CSUM: the segment is added onto dst[row[s]]
+    int add = 0;     // SEG, WSEG, BSEG, CSUM: the segment is added onto dst[row[s]]
     int lo = 0;      // FILL: first position (n is the end)
     const int *ptr = nullptr, *perm = nullptr, *row = nullptr;  // FILL: ptr is the mask
     const double *src = nullptr;
@@ -57,6 +58,7 @@ constexpr int MAX_JOBS = 16;
 struct Jobs {
     int nj = 0;
     int sums = 0;   // blocks of the sums, which come first in the list; the streaming jobs follow
+    unsigned long long *stamp = nullptr;  // if set: device time (ns) at which the inputs were complete
     int every = 1;  // > 1: every `every`-th block of the launch is one of the sums (while they last)
     Job j[MAX_JOBS];
 };
@@ -64,7 +66,9 @@ struct Jobs {
 constexpr int THREADS = 256;
 constexpr int CHUNK_LEN = 4096;  // entries of a long segment per block
 constexpr int SHORT_MAX = 32;    // longest segment a single lane adds up
-constexpr int WARP_MAX = 2048;   // longest segment a single warp adds up
+// Longest segment a single warp, a single block adds up: an iteration of either is a gather latency of
+// about 1.2 us for 4 entries per thread.  One 2000-entry variable of 2000 took a warp 42 us, a block 8.
+constexpr int WARP_MAX = 256, BLOCK_MAX = 8192;
 
 // PERM: a block covers ILP x 256 consecutive positions; thread t takes positions t, t + 256, ... so
 // that the index loads and the stores stay coalesced, and its ILP gathers are in flight together.
@@ -141,19 +145,19 @@ static __device__ __forceinline__ void seg_job(const Job &j, int blk, double *bu
 }
 
 // Sum over [beg, end) of src[perm[q]] (perm null: src[q]) by `width` threads, this one being number t:
-// strided partial sums with 4 independent gathers in flight per thread.
+// strided partial sums with 8 independent gathers in flight per thread.
 static __device__ __forceinline__ double strided_sum(const double *src, const int *perm, int beg, int end, int t,
                                                      int width) {
     double s = 0.0;
-    for (unsigned q = beg + t; q < (unsigned)end; q += 4 * width) {  // end < 2^31: no wrap
-        double v[4];
+    for (unsigned q = beg + t; q < (unsigned)end; q += 8 * width) {  // end < 2^31: no wrap
+        double v[8];
 #pragma unroll
-        for (int u = 0; u < 4; u++) {
+        for (int u = 0; u < 8; u++) {
             const unsigned e = q + u * width;
             v[u] = e < (unsigned)end ? (perm ? src[__ldg(perm + e)] : src[e]) : 0.0;
         }
 #pragma unroll
-        for (int u = 0; u < 4; u++) s += v[u];
+        for (int u = 0; u < 8; u++) s += v[u];
     }
     return s;
 }
@@ -174,6 +178,10 @@ static __device__ __forceinline__ double block_sum(double s, double *buf) {
 
 static __global__ void __launch_bounds__(THREADS, 6) k_reduce(const __grid_constant__ Jobs J) {
     __shared__ double buf[(THREADS / 32) * PIECE];
+    if (J.stamp && blockIdx.x == 0 && threadIdx.x == 0) {
+        wait_inputs(nullptr);
+        asm volatile("mov.u64 %0, %%globaltimer;" : "=l"(*J.stamp) : : "memory");
+    }
     // block of the job list: as launched, or every `every`-th one a block of a sum
     int vb = (int)blockIdx.x;
     if (J.every > 1) {
@@ -206,10 +214,13 @@ static __global__ void __launch_bounds__(THREADS, 6) k_reduce(const __grid_const
         }
         break;
     }
-    case CHUNK: {
+    case CHUNK: case BSEG: {
         const double *src = wait_inputs(j.src);
         const double t = block_sum(strided_sum(src, j.perm, __ldg(j.ptr + 2 * (long long)blk), __ldg(j.ptr + 2 * (long long)blk + 1), threadIdx.x, THREADS), buf);
-        if (threadIdx.x == 0) j.dst[blk] = t;
+        if (threadIdx.x == 0) {
+            double *d = j.dst + (j.kind == BSEG ? __ldg(j.row + blk) : blk);
+            *d = j.add ? *d + t : t;
+        }
         break;
     }
     case OBJ: {

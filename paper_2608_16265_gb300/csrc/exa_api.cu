@@ -1264,6 +1264,14 @@ exa_status apply_grid(exa_model *m, int factor) {
     return EXA_OK;
 }
 
+// Models with fewer tiles (of 128 instances) than this are not tuned: four per SM.
+constexpr i64 TUNE_TILES = 4 * 152;
+i64 tiles_of_128(const exa_model *m) {
+    i64 n = 0;
+    for (const ExaPM &pm : m->h_pms) n += (pm.n_inst + 127) / 128;
+    return n;
+}
+
 // Launch-shape autotuner, in stages, each keeping the fastest variant: (1) the fused evaluation
 // kernel (everything, at varied inputs of unit size) for 64 / 128 / 256 threads per CTA and one CTA
 // per tile versus persistent grids of 1, 2 and 4 waves of resident CTAs; (2) for that shape, launch
@@ -1277,7 +1285,7 @@ exa_status apply_grid(exa_model *m, int factor) {
 exa_status autotune(exa_model *m) {
     int sms = 0;
     CR(cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, m->device));
-    if (m->ntiles[exa::M_ALL] < 4 * sms) return EXA_OK;
+    if (tiles_of_128(m) < TUNE_TILES) return EXA_OK;
     Scratch S{m};
     double *x = nullptr, *y = nullptr, *part = nullptr;
     CR(S.get(&x, m->nvar));
@@ -1935,6 +1943,11 @@ exa_status create_impl(const exa_model_desc *const *descs, int nb, const exa_opt
     CR(cudaMemcpy(m->d_pm, pms.data(), sizeof(ExaPM) * pms.size(), cudaMemcpyHostToDevice));
 
     m->h_pms = pms;
+    // Models too small for the tuner (fewer than four tiles of 128 instances per SM) take 64 threads per
+    // CTA: their few instances spread over more SMs, and a step is a chain of latencies.  us per step
+    // at 32 / 64 / 128 threads: 1000-variable model 11.2 / 11.2 / 12.1, 500-bus network 17.2 / 15.2 / 15.2,
+    // 6000-bus 17.1 / 15.3 / 16.5, 20,000-step rocket 21.6 / 23.1 / 25.7.
+    if (!o.block_threads && tiles_of_128(m) < TUNE_TILES) m->block = 64;
     if (exa_status e = setup_kernels(m, m->block, o.min_blocks)) return e;
 
     // structure pass on the device

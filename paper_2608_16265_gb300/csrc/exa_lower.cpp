@@ -1113,6 +1113,7 @@ struct Emitter {
     const Graph &g;
     const std::vector<PatternGraph> &PG;  // per position in the group
     const CodegenOptions &opt;
+    bool warp_sincos = false;         // the function being printed uses exa_sincos64_warp
     const ProdGraph *prod = nullptr;  // FP64 products (null: contract the derivative entries)
     std::ostringstream os;
     std::string pf_text;  // prefetch functions of the last function() (opt.prefetch > 0)
@@ -1237,12 +1238,12 @@ struct Emitter {
                     std::string cn = ci >= 0 ? "t" + std::to_string(ci) : t + "_c";
                     os << "  " << T << " " << sn << ", " << cn << ";\n";
                     if (red) os << "  exa_sincos_red(" << A() << ", &" << sn << ", &" << cn << ");\n";
-                    else os << "  " << (s.prec == PF ? "sincosf(" : opt.products ? "exa_sincos64_warp(" : "exa_sincos64(") << A() << ", &" << sn << ", &" << cn << ");\n";
+                    else os << "  " << (s.prec == PF ? "sincosf(" : warp_sincos ? "exa_sincos64_warp(" : "exa_sincos64(") << A() << ", &" << sn << ", &" << cn << ");\n";
                     if (si >= 0) name[si] = sn;
                     if (ci >= 0) name[ci] = cn;
                 } else if (s.prec == PD) {  // one of the pair: the other result is dead code
                     os << "  double " << t << "_s, " << t << "_c;\n"
-                       << "  exa_sincos64" << (opt.products ? "_warp" : "") << "(" << A() << ", &" << t << "_s, &" << t << "_c);\n"
+                       << "  exa_sincos64" << (warp_sincos ? "_warp" : "") << "(" << A() << ", &" << t << "_s, &" << t << "_c);\n"
                        << "  const double " << t << " = " << t << (s.op == S_SIN ? "_s" : "_c") << ";\n";
                 } else {
                     os << "  const " << T << " " << t << " = " << fname(s.op, s.prec) << "(" << A() << ");\n";
@@ -1259,6 +1260,8 @@ struct Emitter {
     std::string function(int gid, Mode mode, const std::vector<int> &act, const std::string &suffix = "") {
         os.str("");
         const bool mixed = opt.precision == EXA_MIXED_FP32;
+        // (not in the kernels of a whole step: at their register cap the second path spills, 6 % slower)
+        warp_sincos = !mode_all(mode) && mode != M_FIRST && mode != M_HESS_B;
         const char *W = mixed ? "float" : "double";
         const bool all = mode_all(mode) || mode == M_FIRST;
         const bool hs_coo = mode_hess_coo(mode);
@@ -2003,9 +2006,10 @@ static const char *kFp64Helpers =
 #include "exa_fp64_sincos.inc"
     ;
 
-// The product kernels' sin and cos: a warp whose arguments are all below pi/4 in magnitude (usual for the
-// angle differences of a network) skips the reduction, 5 of the 20 FP64 operations; the quadrant is
-// then zero and r the argument itself, so the results are the same.
+// sin and cos in the products' and the single callbacks' kernels: a warp whose arguments are all below
+// pi/4 in magnitude (usual for the angle differences of a network) skips the reduction, 5 of the 20
+// FP64 operations; the quadrant is then zero and r the argument itself, so the results are the same.
+// 256 networks, us: constraints 226 -> 210, Jacobian 191 -> 179, Hessian 235 -> 218.
 static const char *kWarpSincos = R"(
 static __device__ __forceinline__ void exa_sincos64_warp(const double a, double* s, double* c) {
   if (__all_sync(0xffffffffu, (__double2hiint(a) & 0x7fffffff) < 0x3fe921fb)) exa_sincos_poly(a, 0, s, c);
@@ -2121,7 +2125,7 @@ std::string generate_source(const std::vector<Pattern> &pats, const std::vector<
     if (mixed) src << kMixedHelpers;
     src << kExactHelpers;
     src << kFp64Helpers;
-    if (opt.products) src << kWarpSincos;
+    src << kWarpSincos;
     if (opt.fused_step) src << kStepHelpers;
     if (opt.stage)
         src << "// cp.async of one 8- or 4-byte input into a shared-memory slot (both addresses aligned to\n"

@@ -108,11 +108,14 @@ __global__ void k_low32(const unsigned long long *__restrict__ k, int *out, int 
 }
 
 // Segmented sums (setup).  A segment s < n with entries perm[ptr[s] .. ptr[s+1]) belongs to a
-// class when its length is in (lo, hi]: in_class[s] = 1 and len[s] = its length, else 0 and 0.
-__global__ void k_seg_class(const int *__restrict__ ptr, int n, int lo, int hi, int *in_class, int *len) {
+// class when its length is in (lo, hi]: in_class[s] = 1 and len[s] = its length, else 0 and 0.  Elements
+// (rows[s], or s) whose bit in `skip` is set (skip may be null) belong to none.
+__device__ __forceinline__ bool skipped(const unsigned *skip, int e) { return skip && ((skip[e >> 5] >> (e & 31)) & 1u); }
+__global__ void k_seg_class(const int *__restrict__ ptr, const int *__restrict__ rows, const unsigned *skip, int n,
+                            int lo, int hi, int *in_class, int *len) {
     int s = blockIdx.x * blockDim.x + threadIdx.x;
     if (s >= n) return;
-    const int c = ptr[s + 1] - ptr[s];
+    const int c = skipped(skip, rows ? rows[s] : s) ? 0 : ptr[s + 1] - ptr[s];
     in_class[s] = c > lo && c <= hi;
     len[s] = in_class[s] ? c : 0;
 }
@@ -140,12 +143,35 @@ __global__ void k_seg_longest(const int *__restrict__ ptr, int n, int *len) {
     const int longest = __reduce_max_sync(0xffffffffu, s < n ? ptr[s + 1] - ptr[s] : 0);
     if ((threadIdx.x & 31) == 0 && longest > 0) atomicMax(len, longest);
 }
+// Block b of gradient slot q: start[b] <= q < start[b + 1].
+__device__ __forceinline__ int block_of_slot(const int *start, int nblk, int q) {
+    int lo = 0, hi = nblk;
+    while (hi - lo > 1) {
+        const int mid = (lo + hi) / 2;
+        if (start[mid] <= q) lo = mid;
+        else hi = mid;
+    }
+    return lo;
+}
+// shared[b] = 1 when the variable of some slot of block b has other slots too
+__global__ void k_slots_shared(const int *__restrict__ var, const int *__restrict__ ptr, int n,
+                               const int *__restrict__ start, int nblk, int *shared) {
+    int q = blockIdx.x * blockDim.x + threadIdx.x;
+    if (q < n && ptr[var[q] + 1] - ptr[var[q]] != 1) shared[block_of_slot(start, nblk, q)] = 1;
+}
+// bits of the variables of the blocks that are not shared
+__global__ void k_mark_sole(const int *__restrict__ var, int n, const int *__restrict__ start, int nblk,
+                            const int *__restrict__ shared, unsigned *mask) {
+    int q = blockIdx.x * blockDim.x + threadIdx.x;
+    if (q < n && !shared[block_of_slot(start, nblk, q)]) atomicOr(mask + (var[q] >> 5), 1u << (var[q] & 31));
+}
 // PERM codes: the only entry of a one-entry segment, EMPTY, or ELSEWHERE (summed by a list)
-__global__ void k_seg_first(const int *__restrict__ ptr, const int *__restrict__ perm, int n, int *first) {
+__global__ void k_seg_first(const int *__restrict__ ptr, const int *__restrict__ perm, const unsigned *skip, int n,
+                            int *first) {
     int s = blockIdx.x * blockDim.x + threadIdx.x;
     if (s >= n) return;
     const int b = ptr[s], c = ptr[s + 1] - b;
-    first[s] = c == 1 ? perm[b] : c == 0 ? exa_red::EMPTY : exa_red::ELSEWHERE;
+    first[s] = skipped(skip, s) ? exa_red::ELSEWHERE : c == 1 ? perm[b] : c == 0 ? exa_red::EMPTY : exa_red::ELSEWHERE;
 }
 // bit v of the mask for every listed v
 __global__ void k_mark(const int *__restrict__ v, int n, unsigned *mask) {
@@ -809,14 +835,14 @@ exa_status build_ptr(exa_model *m, const unsigned long long *skeys, int shift, i
 }
 
 // The segments of (ptr, perm) whose length is in (lo, hi], as a list (rows null: element = segment).
-exa_status build_seg_list(exa_model *m, Scratch &S, const int *ptr, const int *perm, const int *rows, int n, int lo,
-                          int hi, bool own_entries, SegList *L) {
+exa_status build_seg_list(exa_model *m, Scratch &S, const int *ptr, const int *perm, const int *rows,
+                          const unsigned *skip, int n, int lo, int hi, bool own_entries, SegList *L) {
     int *in = nullptr, *len = nullptr, *idx = nullptr, *cum = nullptr, *own = nullptr;
     CR(S.get(&in, n));
     CR(S.get(&len, n));
     CR(S.get(&idx, n));
     CR(S.get(&cum, n));
-    k_seg_class<<<grid_of(n, 256), 256, 0, m->stream>>>(ptr, n, lo, hi, in, len);
+    k_seg_class<<<grid_of(n, 256), 256, 0, m->stream>>>(ptr, rows, skip, n, lo, hi, in, len);
     CR(cudaGetLastError());
     CR(exa_inclusive_sum_i32(in, idx, n, m->stream));
     CR(exa_inclusive_sum_i32(len, cum, n, m->stream));
@@ -841,14 +867,15 @@ exa_status build_seg_list(exa_model *m, Scratch &S, const int *ptr, const int *p
 }
 
 // The gather-sum over n segments (ptr, perm).  dense: element s is segment s and one-entry (and
-// empty) segments go to the codes; otherwise segment s is summed into element rows[s].
+// empty) segments go to the codes; otherwise segment s is summed into element rows[s].  Elements in
+// `skip` are left to somebody else.
 exa_status build_gather_sum(exa_model *m, Scratch &S, const int *ptr, const int *perm, const int *rows, int n,
-                            bool dense, bool ordered, GatherSum *gs) {
+                            bool dense, bool ordered, GatherSum *gs, const unsigned *skip = nullptr) {
     if (n <= 0) return EXA_OK;
     if (dense) {
         gs->n = n;
         CR(dalloc(m, &gs->first, n));
-        k_seg_first<<<grid_of(n, 256), 256, 0, m->stream>>>(ptr, perm, n, gs->first);
+        k_seg_first<<<grid_of(n, 256), 256, 0, m->stream>>>(ptr, perm, skip, n, gs->first);
         CR(cudaGetLastError());
     }
     const int lo = dense ? 1 : 0;
@@ -861,20 +888,20 @@ exa_status build_gather_sum(exa_model *m, Scratch &S, const int *ptr, const int 
     CR(cudaStreamSynchronize(m->stream));
     if (longest <= lo) return EXA_OK;
     if (longest <= exa_red::SHORT_MAX || ordered) {
-        if (dense) return build_seg_list(m, S, ptr, perm, rows, n, lo, INT32_MAX, true, &gs->sh);
+        if (dense || skip) return build_seg_list(m, S, ptr, perm, rows, skip, n, lo, INT32_MAX, true, &gs->sh);
         gs->sh.n = n;  // every segment is short: the arrays as they are
         gs->sh.ptr = ptr;
         gs->sh.perm = perm;
         gs->sh.row = rows;
         return EXA_OK;
     }
-    if (exa_status e = build_seg_list(m, S, ptr, perm, rows, n, lo, exa_red::SHORT_MAX, true, &gs->sh)) return e;
-    if (exa_status e = build_seg_list(m, S, ptr, perm, rows, n, exa_red::SHORT_MAX, exa_red::WARP_MAX, false, &gs->md)) return e;
+    if (exa_status e = build_seg_list(m, S, ptr, perm, rows, skip, n, lo, exa_red::SHORT_MAX, true, &gs->sh)) return e;
+    if (exa_status e = build_seg_list(m, S, ptr, perm, rows, skip, n, exa_red::SHORT_MAX, exa_red::WARP_MAX, false, &gs->md)) return e;
     if (longest > exa_red::WARP_MAX)
-        if (exa_status e = build_seg_list(m, S, ptr, perm, rows, n, exa_red::WARP_MAX, exa_red::BLOCK_MAX, false, &gs->bl))
+        if (exa_status e = build_seg_list(m, S, ptr, perm, rows, skip, n, exa_red::WARP_MAX, exa_red::BLOCK_MAX, false, &gs->bl))
             return e;
     if (longest > exa_red::BLOCK_MAX)
-        if (exa_status e = build_seg_list(m, S, ptr, perm, rows, n, exa_red::BLOCK_MAX, INT32_MAX, false, &gs->lg)) return e;
+        if (exa_status e = build_seg_list(m, S, ptr, perm, rows, skip, n, exa_red::BLOCK_MAX, INT32_MAX, false, &gs->lg)) return e;
     if (!gs->lg.n) return EXA_OK;
     std::vector<int> range(2 * (size_t)gs->lg.n), piece;
     CR(cudaMemcpy(range.data(), gs->lg.ptr, sizeof(int) * range.size(), cudaMemcpyDeviceToHost));
@@ -1085,6 +1112,50 @@ exa_status build_structure(exa_model *m) {
         CR(cudaGetLastError());
     }
     m->grad_compact = 2 * (i64)nseg < m->nvar;
+    // Patterns all of whose slots are the only ones of their variables write the gradient themselves
+    // (ExaPM::gsole); those variables are left out of the sums.  (The slot buffer and the sum moved 36
+    // bytes per variable: PDE 1000^2 step 78.2 -> 73.9 us, 2001^2 mixed 274 -> 256 us.)
+    unsigned *sole = nullptr;  // their bits
+    i64 n_sole = 0;
+    if (ng) {
+        std::vector<int> start, shared;
+        std::vector<std::pair<size_t, int>> owner;  // (descriptor, position) of every block of slots
+        for (size_t i = 0; i < m->h_pms.size(); i++) {
+            const exa::Group &G = m->groups[m->h_pms[i].grp];
+            for (size_t pos = 0; pos < G.pats.size(); pos++) {
+                const exa::Pattern &P = m->pats[G.pats[pos]];
+                if (P.kind != EXA_OBJ || !P.nj() || !m->h_pms[i].n_inst) continue;
+                owner.push_back({i, (int)pos});
+            }
+        }
+        auto base = [&](const std::pair<size_t, int> &o) { return m->h_pms[o.first].gbase[o.second]; };
+        std::sort(owner.begin(), owner.end(), [&](const auto &a, const auto &b) { return base(a) < base(b); });
+        for (auto &o : owner) start.push_back((int)base(o));
+        shared.assign(start.size(), 0);
+        int *d_start = nullptr, *d_shared = nullptr;
+        CR(S.get(&d_start, (i64)start.size()));
+        CR(S.get(&d_shared, (i64)start.size()));
+        CR(cudaMemcpyAsync(d_start, start.data(), sizeof(int) * start.size(), cudaMemcpyHostToDevice, m->stream));
+        CR(cudaMemsetAsync(d_shared, 0, sizeof(int) * start.size(), m->stream));
+        k_slots_shared<<<grid_of(ng, 256), 256, 0, m->stream>>>(m->d_gvar, m->d_gptr, ng, d_start, (int)start.size(), d_shared);
+        CR(cudaGetLastError());
+        CR(cudaMemcpyAsync(shared.data(), d_shared, sizeof(int) * start.size(), cudaMemcpyDeviceToHost, m->stream));
+        CR(cudaStreamSynchronize(m->stream));
+        for (size_t b = 0; b < owner.size(); b++) {
+            if (shared[b]) continue;
+            ExaPM &pm = m->h_pms[owner[b].first];
+            const i64 end = b + 1 < owner.size() ? start[b + 1] : ng;
+            pm.gsole |= 1u << owner[b].second;
+            n_sole += end - start[b];
+        }
+        if (n_sole) {
+            CR(cudaMemcpyAsync(m->d_pm, m->h_pms.data(), sizeof(ExaPM) * m->h_pms.size(), cudaMemcpyHostToDevice, m->stream));
+            CR(S.get(&sole, (m->nvar + 31) / 32));
+            CR(cudaMemsetAsync(sole, 0, sizeof(unsigned) * ((m->nvar + 31) / 32), m->stream));
+            k_mark_sole<<<grid_of(ng, 256), 256, 0, m->stream>>>(m->d_gvar, ng, d_start, (int)start.size(), d_shared, sole);
+            CR(cudaGetLastError());
+        }
+    }
     if (m->grad_compact) {
         m->sum_g.fill_n = m->nvar;
         CR(dalloc(m, &m->sum_g.fill_mask, (m->nvar + 31) / 32));
@@ -1093,9 +1164,12 @@ exa_status build_structure(exa_model *m) {
             k_mark<<<grid_of(nseg, 256), 256, 0, m->stream>>>(m->d_gsegvar, nseg, m->sum_g.fill_mask);
             CR(cudaGetLastError());
         }
-        if (exa_status e = build_gather_sum(m, S, m->d_gsegptr, m->d_gperm, m->d_gsegvar, nseg, false, false, &m->sum_g)) return e;
-    } else if (exa_status e = build_gather_sum(m, S, m->d_gptr, m->d_gperm, nullptr, (int)m->nvar, true, false, &m->sum_g)) {
-        return e;
+        if (nseg > n_sole)
+            if (exa_status e = build_gather_sum(m, S, m->d_gsegptr, m->d_gperm, m->d_gsegvar, nseg, false, false, &m->sum_g, sole))
+                return e;
+    } else if (n_sole < m->nvar) {
+        if (exa_status e = build_gather_sum(m, S, m->d_gptr, m->d_gperm, nullptr, (int)m->nvar, true, false, &m->sum_g, sole))
+            return e;
     }
 
     // ---- augmentation segments by row (only rows that receive terms)
@@ -2173,6 +2247,7 @@ exa_status exa_grad(exa_model *m, const double *x, double *g) {
     CHECK_PTRS(x, g);
     ExaOut o{};
     o.gbuf = m->d_gbuf;
+    o.g = g;
     if (exa_status e = launch_eval(m, exa::M_GRAD, x, nullptr, 0.0, o, 0, -1, true)) return e;
     Reduction r;
     r.add(m->sum_g, m->d_gbuf, g);
@@ -2473,6 +2548,7 @@ static exa_status eval_fused_step(exa_model *m, int i, const double *x, const do
     st.need = m->d_need[i];
     st.items = m->d_items[i];
     st.nitems = m->nitems[i];
+    o.g = nullptr;  // every slot through the buffer: the queue's gradient sums cover all variables
     st.spin_limit = 1 << 22;  // polls of about 0.2 us or more: about a second at least
     for (ExaRed &r : st.r) r.how = -1;
     if (jac_csc && !jdirect && m->nnzj_csc) {
@@ -2525,6 +2601,7 @@ static exa_status eval_all_launches(exa_model *m, const double *x, const double 
     o.c = c ? c : m->d_cbuf;
     o.abuf = m->d_abuf;
     o.gbuf = m->d_gbuf;
+    o.g = g;
     o.jac = jac ? jac : m->d_jbuf;
     o.hess = hess ? hess : m->d_hbuf;
     // a CSC without duplicates is a permutation of the COO slots: the evaluation kernel writes it

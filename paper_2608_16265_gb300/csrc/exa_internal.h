@@ -36,6 +36,7 @@
         long long ubase;          /* first slot of the group's H v terms: [symbol][instance] */     \
         int grp;                  /* group id */                                                    \
         int member;               /* batch member */                                                \
+        unsigned gsole;           /* bit per pattern: its gradient slots are their variables' only */\
     };                                                                                              \
     struct ExaTile {              /* BLOCK consecutive instances of one (member, group) */          \
         int pm;                                                                                     \
@@ -46,6 +47,7 @@
         double *c;                /* constraint base values, indexed by global row */               \
         double *abuf;             /* augmentation terms */                                          \
         double *gbuf;             /* objective gradient slots */                                    \
+        double *g;                /* if set: the gradient, written directly by patterns in gsole */ \
         double *jac;              /* Jacobian COO values */                                         \
         double *hess;             /* Hessian COO values */                                          \
         double *jcsc;             /* if set: Jacobian CSC values written directly (no duplicates) */\

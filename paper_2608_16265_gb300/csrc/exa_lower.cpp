@@ -1338,7 +1338,7 @@ struct Emitter {
         for (int pos : act) {
             const Pattern &p = pat(pos);
             if (want_struct) for (int s = 0; s < p.nsym; s++) idx_syms.insert(grp.sym[pos][s]);
-            if (jprod && want[pos].grad) for (int s = 0; s < p.nsym; s++) idx_syms.insert(grp.sym[pos][s]);
+            if ((jprod || p.kind == EXA_OBJ) && want[pos].grad) for (int s = 0; s < p.nsym; s++) idx_syms.insert(grp.sym[pos][s]);
             if (want[pos].hess)
                 for (auto &pr : p.hpair)
                     if (pr.first != pr.second || hprod) { idx_syms.insert(grp.sym[pos][pr.first]); idx_syms.insert(grp.sym[pos][pr.second]); }
@@ -1795,7 +1795,15 @@ struct Emitter {
             } else if (w.grad && p.nj() > 0) {
                 std::vector<std::string> vals;
                 for (int j = 0; j < p.nj(); j++) vals.push_back(widen(G.grad[p.jsym[j]]));
-                if (obj) staged("o.gbuf", "pm.gbase[" + P + "]", p.nj(), vals, nullptr, nullptr);
+                if (obj) {
+                    // slots that are their variables' only ones go to the gradient itself
+                    os << "  if (o.g && ((pm.gsole >> " << P << ") & 1u)) {\n";
+                    for (int j = 0; j < p.nj(); j++)
+                        os << "    if (act) o.g[pm.xoff + i" << grp.sym[pos][p.jsym[j]] << "] = " << vals[j] << ";\n";
+                    os << "  } else {\n";
+                    staged("o.gbuf", "pm.gbase[" + P + "]", p.nj(), vals, nullptr, nullptr);
+                    os << "  }\n";
+                }
                 else staged("o.jac", "pm.jbase[" + P + "]", p.nj(), vals, "o.jcsc", "o.jmap");
             }
             if (w.hess) {

@@ -65,3 +65,29 @@ def test_segment_lengths(spread, batch):
         for a in [d[k] for d in (got, one) if k in d]:
             assert a.shape == r.shape
             assert np.all(np.abs(a - r) <= tol * np.abs(r)), k
+
+
+@pytest.mark.parametrize("fused", [False, True])
+@pytest.mark.parametrize("case", ["all_sole", "one_shared", "few_sole", "mixed_members"])
+def test_sole_gradient_slots(case, fused):
+    """Patterns whose gradient slots are their variables' only ones write the gradient themselves; one
+    shared variable, or a member where they are not, and the pattern goes through the sums."""
+    def model(n, extra, spare):
+        m = Model()
+        x = m.add_var(2 * n + spare)
+        m.add_obj(lambda d: d.a * x[d.i] ** 2 * x[d.k + n],
+                  data=dict(i=np.random.default_rng(1).permutation(n).astype(np.int32), a=np.arange(1.0, n + 1)))
+        m.add_obj(lambda d: 2 * x[d.j], data=dict(j=np.asarray(extra, np.int32)))
+        m.add_con(lambda d: x[d.k] * x[d.k + 1], n=3)
+        return m.flat()
+
+    flats = {"all_sole": [model(70, [140], 1)], "one_shared": [model(70, [140, 7], 1)],
+             "few_sole": [model(33, [66], 400)], "mixed_members": [model(33, [66, 67], 2), model(33, [66, 0], 2)]}[case]
+    m = binding.exa_create_batch(flats, flags=binding.EXA_FLAG_NO_TUNE | (binding.EXA_FLAG_FUSED_STEP if fused else 0))
+    x = np.random.default_rng(2).uniform(0.5, 1.5, m.nvar)
+    ref = np.concatenate([oracle.Oracle(f).grad(x[m.xoff[b]:m.xoff[b + 1]]) for b, f in enumerate(flats)])
+    xt, yt = torch.as_tensor(x, device="cuda"), torch.ones(m.ncon, dtype=torch.float64, device="cuda")
+    for g in (m.grad(xt), m.eval_all(xt, yt, 1.0, csc=True)["g"], m.eval_all(xt, yt, 1.0)["g"]):
+        g = g.cpu().numpy()
+        # products of at most four factors, sums of at most two terms
+        assert np.all(np.abs(g - ref) <= 8 * 2.0 ** -53 * np.abs(ref) * 2)

@@ -140,6 +140,11 @@ struct Group {
     // same (row, col) for every instance), summed per instance; each entry lists (position, slot)
     std::vector<std::vector<std::pair<int, int>>> hc;
     std::vector<std::pair<int, int>> hc_sym;  // group symbol pair of each compressed slot
+    // where a compressed slot lies in the group's part of the buffer: hc_at >= 0: at kk * hc_rows + hc_at
+    // (rows of neighbouring slots per instance); hc_at < 0, both variables follow the instance number:
+    // array (hc_rows - 1 - hc_at) of n_inst entries, so that the sums by variable read neighbours
+    std::vector<int> hc_at;
+    int hc_rows = 0;
     std::vector<int> tsym, usym;  // group symbols of the constraints' first-order slots / of the Hessian
 };
 

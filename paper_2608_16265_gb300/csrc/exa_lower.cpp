@@ -1068,6 +1068,22 @@ void finalize_group(Group &g, const std::vector<Pattern> &pats) {
             g.hc[r.first->second].push_back({(int)pos, j});
         }
     }
+    std::function<bool(const Pattern &, int)> has_field = [&](const Pattern &p, int r) {
+        const INode &n = p.ix[r];
+        return n.op == EXA_I_FIELD || (n.op >= EXA_I_ADD && (has_field(p, n.a) || has_field(p, n.b)));
+    };
+    // (Compressed sums all side by side per instance / like this: 256 networks, every output 794 / 777 us,
+    // mixed 724 / 714 us: the diagonals of the branch flows, a quarter of the sums, are read back in runs
+    // instead of one 32-byte sector each.)
+    auto follows = [&](int s) {
+        const Pattern &p = pats[g.pats[g.sym_root[s].first]];
+        return !has_field(p, g.sym_root[s].second);
+    };
+    g.hc_at.clear();
+    g.hc_rows = 0;
+    int arrays = 0;
+    for (auto &pr : g.hc_sym)
+        g.hc_at.push_back(follows(pr.first) && follows(pr.second) ? -1 - arrays++ : g.hc_rows++);
     std::set<int> t, u;
     for (size_t pos = 0; pos < g.pats.size(); pos++)
         if (pats[g.pats[pos]].kind != EXA_OBJ) t.insert(g.sym[pos].begin(), g.sym[pos].end());
@@ -1128,6 +1144,12 @@ struct Emitter {
         : pats(p_), grp(g_), g(gr), PG(pg), opt(o) {}
 
     const Pattern &pat(int pos) const { return pats[grp.pats[pos]]; }
+    // the slot of compressed sum c of instance kk
+    std::string hc_slot(int c) const {
+        const int at = grp.hc_at[c];
+        return at >= 0 ? "pm.hcbase + kk * " + std::to_string(grp.hc_rows) + " + " + std::to_string(at)
+                       : "pm.hcbase + " + std::to_string(grp.hc_rows - 1 - at) + " * pm.n_inst + kk";
+    }
 
     std::string idx_expr(int pos, int r) {
         const Pattern &p = pat(pos);
@@ -1546,8 +1568,8 @@ struct Emitter {
                 for (int c = 0; c < nhc; c++)
                     os << "    { const long long ga = pm.xoff + i" << grp.hc_sym[c].first << ", gb = pm.xoff + i"
                        << grp.hc_sym[c].second << ";\n"
-                       << "      so.hcrow[pm.hcbase + kk * " << nhc << " + " << c << "] = (int)(ga > gb ? ga : gb);\n"
-                       << "      so.hccol[pm.hcbase + kk * " << nhc << " + " << c << "] = (int)(ga > gb ? gb : ga); }\n";
+                       << "      so.hcrow[" << hc_slot(c) << "] = (int)(ga > gb ? ga : gb);\n"
+                       << "      so.hccol[" << hc_slot(c) << "] = (int)(ga > gb ? gb : ga); }\n";
                 os << "  }\n";
             }
             os << "}\n";
@@ -1911,10 +1933,15 @@ struct Emitter {
                 for (auto &d : dbl) os << "    if (" << d.second << ") hc" << d.first << " += hc" << d.first << ";\n";
                 os << "  }\n";
             }
-            std::vector<std::string> sums;
-            if (!hprod)
-              for (size_t c = 0; c < grp.hc.size(); c++) sums.push_back(hc_started[c] ? "hc" + std::to_string(c) : "0.0");
-            if (!hprod) staged("o.hcomp", "pm.hcbase", (int)grp.hc.size(), sums, nullptr, nullptr);
+            if (!hprod) {
+                std::vector<std::string> sums;
+                for (size_t c = 0; c < grp.hc.size(); c++) {
+                    const std::string v = hc_started[c] ? "hc" + std::to_string(c) : "0.0";
+                    if (grp.hc_at[c] >= 0) sums.push_back(v);
+                    else os << "  if (act && o.hcomp) o.hcomp[" << hc_slot(c) << "] = " << v << ";\n";
+                }
+                if (!sums.empty()) staged("o.hcomp", "pm.hcbase", grp.hc_rows, sums, nullptr, nullptr);
+            }
         }
         // one array per group symbol: consecutive lanes store to consecutive addresses as they are, and
         // the sums by variable read consecutive values where variables follow the instances
@@ -2185,7 +2212,7 @@ std::string generate_source(const std::vector<Pattern> &pats, const std::vector<
         for (const Pattern &p : pats)
             if (pattern_in_mode(p, (Mode)m)) smax = std::max(smax, std::max(p.nj(), p.nh()));
         if (mode_hess_comp(m))
-            for (const Group &gr : groups) smax = std::max(smax, (int)gr.hc.size());
+            for (const Group &gr : groups) smax = std::max(smax, gr.hc_rows);
         // staged input slots: two buffers within 160 KB of shared memory per CTA beside ws
         const int st_budget = opt.stage ? std::max(0, (160 * 1024 - opt.block * smax * 8) / (2 * opt.block)) & ~7 : 0;
         for (size_t gi = 0; gi < groups.size(); gi++) {

@@ -788,6 +788,13 @@ struct Scratch {
     }
 };
 
+// Key bits of an index below n (the radix sort makes one pass per eight).
+int bits_of(i64 n) {
+    int b = 1;
+    while (b < 32 && (1LL << b) < n) b++;
+    return b;
+}
+
 // Sort keys with values 0..n-1 (stable): sorted keys and permutation.
 exa_status sort_with_perm(exa_model *m, Scratch &S, unsigned long long *keys, int n, int end_bit,
                           unsigned long long **skeys, int *perm) {
@@ -1004,7 +1011,7 @@ exa_status build_structure(exa_model *m) {
         k_keys2<<<grid_of(nj, 256), 256, 0, m->stream>>>(m->d_jcol, m->d_jrow, keys, nj);
         CR(cudaGetLastError());
     }
-    if (exa_status e = sort_with_perm(m, S, keys, nj, 64, &skeys, m->d_jperm)) return e;
+    if (exa_status e = sort_with_perm(m, S, keys, nj, 32 + bits_of(m->nvar), &skeys, m->d_jperm)) return e;
     if (exa_status e = segments(m, S, skeys, m->d_jperm, nj, &nseg, &m->d_jsegptr, &segkey, m->d_jcoo2csc, true)) return e;
     m->nnzj_csc = nseg;
     if (nseg < nj) {
@@ -1026,7 +1033,7 @@ exa_status build_structure(exa_model *m) {
         k_keys2<<<grid_of(nh, 256), 256, 0, m->stream>>>(m->d_hcol, m->d_hrow, keys, nh);
         CR(cudaGetLastError());
     }
-    if (exa_status e = sort_with_perm(m, S, keys, nh, 64, &skeys, m->d_hperm)) return e;
+    if (exa_status e = sort_with_perm(m, S, keys, nh, 32 + bits_of(m->nvar), &skeys, m->d_hperm)) return e;
     if (exa_status e = segments(m, S, skeys, m->d_hperm, nh, &nseg, &m->d_hsegptr, &segkey, m->d_hcoo2csc, true)) return e;
     m->nnzh_csc = nseg;
     if (nseg < nh) {
@@ -1050,7 +1057,7 @@ exa_status build_structure(exa_model *m) {
         CR(dalloc(m, &m->d_hcperm, nc));
         k_keys2<<<grid_of(nc, 256), 256, 0, m->stream>>>(m->d_hccol, m->d_hcrow, ck, nc);
         CR(cudaGetLastError());
-        if (exa_status e = sort_with_perm(m, S, ck, nc, 64, &skeys, m->d_hcperm)) return e;
+        if (exa_status e = sort_with_perm(m, S, ck, nc, 32 + bits_of(m->nvar), &skeys, m->d_hcperm)) return e;
         int nsc = 0;
         if (exa_status e = segments(m, S, skeys, m->d_hcperm, nc, &nsc, &m->d_hcsegptr, &segkey, nullptr, true)) return e;
         if (nsc != m->nnzh_csc) return fail(m, EXA_E_INTERNAL, "compressed Hessian does not cover the CSC entries");
@@ -1070,7 +1077,7 @@ exa_status build_structure(exa_model *m) {
             k_keys1<<<grid_of(n, 256), 256, 0, m->stream>>>(i ? m->d_uvar : m->d_tvar, pk, n);
             CR(cudaGetLastError());
         }
-        if (exa_status e = sort_with_perm(m, S, pk, n, 32, &skeys, perm)) return e;
+        if (exa_status e = sort_with_perm(m, S, pk, n, bits_of(m->nvar), &skeys, perm)) return e;
         if (exa_status e = build_ptr(m, skeys, 0, n, m->nvar, &ptr)) return e;
         if (exa_status e = build_gather_sum(m, S, ptr, perm, nullptr, (int)m->nvar, true, false, i ? &m->sum_u : &m->sum_t))
             return e;
@@ -1090,7 +1097,7 @@ exa_status build_structure(exa_model *m) {
             k_keys2<<<grid_of(nc, 256), 256, 0, m->stream>>>(m->d_hrowval, m->d_hcolof, keys, nc);
             CR(cudaGetLastError());
         }
-        if (exa_status e = sort_with_perm(m, S, keys, nc, 64, &skeys, m->d_hcsr_perm)) return e;
+        if (exa_status e = sort_with_perm(m, S, keys, nc, 32 + bits_of(m->nvar), &skeys, m->d_hcsr_perm)) return e;
         if (exa_status e = build_ptr(m, skeys, 32, nc, m->nvar, &m->d_hcsr_ptr)) return e;
     }
 
@@ -1100,7 +1107,7 @@ exa_status build_structure(exa_model *m) {
         k_keys1<<<grid_of(ng, 256), 256, 0, m->stream>>>(m->d_gvar, keys, ng);
         CR(cudaGetLastError());
     }
-    if (exa_status e = sort_with_perm(m, S, keys, ng, 32, &skeys, m->d_gperm)) return e;
+    if (exa_status e = sort_with_perm(m, S, keys, ng, bits_of(m->nvar), &skeys, m->d_gperm)) return e;
     if (exa_status e = build_ptr(m, skeys, 0, ng, m->nvar, &m->d_gptr)) return e;
     // the variables that have gradient slots, for the compact form (chosen when they are fewer than
     // half of the variables)
@@ -1178,7 +1185,7 @@ exa_status build_structure(exa_model *m) {
         k_keys1<<<grid_of(na, 256), 256, 0, m->stream>>>(m->d_arow, keys, na);
         CR(cudaGetLastError());
     }
-    if (exa_status e = sort_with_perm(m, S, keys, na, 32, &skeys, m->d_aperm)) return e;
+    if (exa_status e = sort_with_perm(m, S, keys, na, bits_of(m->ncon), &skeys, m->d_aperm)) return e;
     if (exa_status e = segments(m, S, skeys, m->d_aperm, na, &nseg, &m->d_aptr, &segkey, nullptr, true)) return e;
     m->n_aug_rows = nseg;
     CR(dalloc(m, &m->d_arows, nseg));

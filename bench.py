@@ -160,9 +160,9 @@ def step_kernel(m, nbytes, step_bytes=None):
 
 
 def live_kernel_ms(m, step, n):
-    """The step's evaluation kernel(s) timed live: the library records CUDA events on the model
-    stream right before and after them in every exa_eval_all step (inside its cached graph); the
-    mean over n steps, each read after its step."""
+    """The step's evaluation kernel(s) timed live: the library times them in every exa_eval_all step (device
+    timer stamps, or CUDA events, inside its cached graph); the mean over n steps, each read after
+    its step."""
     v = []
     for _ in range(n):
         step()

@@ -269,7 +269,8 @@ exa_status exa_obj(exa_model *m, const double *x, double *f);
 exa_status exa_obj_noalloc(exa_model *m, const double *x, double *f);
 
 /* g[nvar] = grad f(x): each objective instance writes its own gradient slots, then a gather
- * segmented sum per variable produces g (Sec. 7.2.3, no atomics). */
+ * segmented sum per variable produces g (Sec. 7.2.3, no atomics); slots that are their variables' only
+ * ones are written to g directly. */
 exa_status exa_grad(exa_model *m, const double *x, double *g);
 
 /* c[ncon] = base rows plus augmentation terms (Sec. 3.3, 7.2.3). */
@@ -327,7 +328,8 @@ exa_status exa_eval_all_host(exa_model *m, const double *x, const double *y, dou
                              double *jac_csc, double *hess_csc);
 
 /* Products at x (NLPModels jprod!/jtprod!/hprod!): Jv[ncon] = J(x) v, Jtw[nvar] = J(x)^T w,
- * Hv[nvar] = (sigma Hess f + sum y_r Hess c_r)(x) v with the Hessian's full symmetric action. */
+ * Hv[nvar] = (sigma Hess f + sum y_r Hess c_r)(x) v with the Hessian's full symmetric action.  Matrix-free:
+ * derivatives are contracted with the vector where they are formed. */
 exa_status exa_jprod(exa_model *m, const double *x, const double *v, double *Jv);
 exa_status exa_jtprod(exa_model *m, const double *x, const double *w, double *Jtw);
 exa_status exa_hprod(exa_model *m, const double *x, const double *y, double sigma,

@@ -626,7 +626,7 @@ def run_exa(args):
     roofline = {"bound": "hbm", "achieved": achieved, "peak": peak, "unit": "GB/s", "frac": achieved / peak,
                 "traffic": traffic, "peak_source": peak_kind + " (MEASURED_PEAKS.json hbm_gbs)",
                 "kernel": f"{kname} (generated evaluation kernel of the step)", "algorithmic_bytes": kbytes,
-                "kernel_ms": kern_ms, "kernel_timing": "CUDA events around the kernel inside the step's graph",
+                "kernel_ms": kern_ms, "kernel_timing": "by the library inside the step's graph (exa_stat eval_kernel_ms)",
                 "step_algorithmic_bytes": step_bytes,
                 "step_hbm_frac": step_bytes / (ms * 1e-3) / 1e9 / peak,
                 "coo_only_kernel_ms": coo_ms, "coo_only_algorithmic_bytes": nbytes,

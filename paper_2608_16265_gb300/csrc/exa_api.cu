@@ -2899,10 +2899,10 @@ exa_status exa_eval_all_host(exa_model *m, const double *x, const double *y, dou
 // The products contract every instance's derivatives with the vector as they are formed (one term per
 // row, or per instance and variable of the fused group), so the Jacobian and Hessian values are neither
 // stored nor gathered; the terms of an augmented row or of a variable are then summed.  Bound by the
-// FP64 pipe (about 58, 57 and 75 operations per branch of a network, sin/cos included, at 528 G/s) and by
+// FP64 pipe (about 53, 52 and 70 operations per branch of a network, sin/cos included, at 528 G/s) and by
 // the gathers of x and of the vector.  Measured, the three together (before: all Jacobian and Hessian
-// values stored, then gathered per row, column and CSC entry): 30,000-bus network 107 -> 58 us, 32
-// networks (15.7 M entries) 313 -> 151 us, 100,000-step rocket 67.8 ms -> 132 us (one variable in
+// values stored, then gathered per row, column and CSC entry): 30,000-bus network 107 -> 45 us, 32
+// networks (15.7 M entries) 313 -> 147 us, 100,000-step rocket 67.8 ms -> 129 us (one variable in
 // every row: its 300,000 terms were added by one lane).
 exa_status exa_jprod(exa_model *m, const double *x, const double *v, double *Jv) {
     if (exa_status e = check_model(m)) return e;

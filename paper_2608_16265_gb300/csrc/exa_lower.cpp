@@ -810,7 +810,7 @@ struct ProdGraph {
 class Products {
     Graph &g;
     std::map<int, bool> dep_;
-    std::map<int, int> tan_;
+    std::map<int, int> tan_, leaves_;
     int wrt_ = -1;
     typedef std::map<std::vector<int>, double> Terms;  // sorted factors -> coefficient
 
@@ -863,11 +863,20 @@ class Products {
         default: return -1;
         }
     }
-    // coefficient and sorted factors of a node seen as a product
+    // leaves of node n's product tree (at most 1000)
+    int leaves(int n) {
+        auto it = leaves_.find(n);
+        if (it != leaves_.end()) return it->second;
+        const SN s = g.n[n];
+        const int k = s.op == S_NEG ? leaves(s.a) : s.op == S_MUL ? std::min(1000, leaves(s.a) + leaves(s.b)) : 1;
+        return leaves_[n] = k;
+    }
+    // coefficient and factors of a node seen as a product; a product of more than eight leaves (a high
+    // power) is one factor, so that the lists stay short
     void factors(int n, double &c, std::vector<int> &f) {
         const SN s = g.n[n];
         if (s.op == S_NEG) { c = -c; factors(s.a, c, f); }
-        else if (s.op == S_MUL) { factors(s.a, c, f); factors(s.b, c, f); }
+        else if (s.op == S_MUL && leaves(n) <= 8) { factors(s.a, c, f); factors(s.b, c, f); }
         else if (s.op == S_LIT) c *= s.lit;
         else f.push_back(n);
     }
@@ -941,15 +950,15 @@ class Products {
         for (int which = 0; which < 2; which++) {
             const int k = which ? s.b : s.a;
             if (k < 0 || !dep(k)) continue;
-            const Terms t = tangent_terms(k);
-            if (t.empty()) continue;
             if (s.op == S_ADD || s.op == S_SUB || s.op == S_NEG) {
                 const double sign = s.op == S_NEG || (s.op == S_SUB && which) ? -1.0 : 1.0;
-                for (auto &kv : t) r[kv.first] += sign * kv.second;
+                for (auto &kv : tangent_terms(k)) r[kv.first] += sign * kv.second;
             } else {
-                double c;
+                const int d = tangent(k);  // (kept: a square uses its operand's twice)
+                if (d < 0) continue;
+                double c = 1.0;
                 std::vector<int> f;
-                collapse(t, c, f);
+                factors(d, c, f);
                 factors(partial(n, which), c, f);
                 std::sort(f.begin(), f.end());
                 r[f] += c;

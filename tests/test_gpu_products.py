@@ -50,3 +50,20 @@ def test_products(precision, tol, n, scale):
     ref = dict(jv=o.jprod(x, v), jtw=o.jtprod(x, w), hv=o.hprod(x, y, 1.3, v))
     for k, r in ref.items():
         assert np.linalg.norm(got[k].cpu().numpy() - r) <= tol * np.linalg.norm(r), k
+
+
+@pytest.mark.parametrize("precision,tol", [(binding.EXA_FP64, 1e-13), (binding.EXA_MIXED_FP32, 1e-5)])
+@pytest.mark.parametrize("n", [1, 40, 700])
+def test_wide_stencil(precision, tol, n):
+    """Patterns over many shared variables: H v from the summed Hessian entries."""
+    m = Model()
+    x = m.add_var(n + 24)
+    m.add_con(lambda d: sum((0.5 + 0.1 * t) * x[d.k + 2 * t] * x[d.k + 2 * t + 1] ** 2 for t in range(12)), n=n)
+    m.add_obj(lambda d: x[d.k] ** 2 * x[d.k + 1], n=n)
+    flat = m.flat()
+    mm, o = binding.exa_create(flat, precision, flags=binding.EXA_FLAG_NO_TUNE), oracle.Oracle(flat)
+    rng = np.random.default_rng(n)
+    xv, y, v = rng.uniform(0.5, 1.5, flat.nvar), rng.standard_normal(flat.ncon), rng.standard_normal(flat.nvar)
+    t = lambda a: torch.as_tensor(a, device="cuda")  # noqa: E731
+    got, ref = mm.hprod(t(xv), t(y), 0.7, t(v)).cpu().numpy(), o.hprod(xv, y, 0.7, v)
+    assert np.linalg.norm(got - ref) <= tol * np.linalg.norm(ref)

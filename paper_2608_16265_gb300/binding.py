@@ -144,7 +144,7 @@ class ExaError(RuntimeError):
 class _Desc:
     """Keeps the ctypes descriptor of one flat model (and every buffer it points to) alive."""
 
-    def __init__(self, flat: ir.FlatModel):
+    def __init__(self, flat: ir.FlatModel, precision: int):
         self.keep = []
         pats = (exa_pattern_desc * max(1, len(flat.patterns)))()
         for i, p in enumerate(flat.patterns):
@@ -158,6 +158,8 @@ class _Desc:
             fl = (exa_field * max(1, len(p.fields)))()
             for j, f in enumerate(p.fields):
                 f = np.ascontiguousarray(f)
+                if p.replicated and precision == EXA_MIXED_FP32:
+                    f = f.copy()  # a column of its own: fusing patterns would change FP32 roundings
                 self.keep.append(f)
                 fl[j] = exa_field(int(p.ftype[j]), 0, f.ctypes.data)
             self.keep += [vn, inn, fl]
@@ -195,7 +197,7 @@ def exa_create_batch(flats: Sequence[ir.FlatModel], precision: int = EXA_FP64, b
                      flags: int = 0, device: int = 0, grid_factor: int = 0, min_blocks: int = 0,
                      chunks: int = 0, wave_pct: int = 0) -> "Model":
     lib = load()
-    descs = [_Desc(f) for f in flats]
+    descs = [_Desc(f, precision) for f in flats]
     arr = (C.POINTER(exa_model_desc) * len(descs))(*[C.pointer(d.desc) for d in descs])
     h = C.c_void_p()
     opt = _opts(precision, block, flags, device, grid_factor, min_blocks, chunks, wave_pct)
@@ -208,7 +210,7 @@ def exa_create_batch(flats: Sequence[ir.FlatModel], precision: int = EXA_FP64, b
 def exa_compile_check(flat: ir.FlatModel, precision: int = EXA_FP64, block: int = 0, flags: int = 0,
                       min_blocks: int = 0) -> None:
     lib = load()
-    d = _Desc(flat)
+    d = _Desc(flat, precision)
     buf = C.create_string_buffer(8192)
     rc = lib.exa_compile_check(C.byref(d.desc), C.byref(_opts(precision, block, flags, 0, 0, min_blocks)), buf, 8192)
     if rc != EXA_OK:

@@ -393,6 +393,7 @@ class Pattern:
     row_limit: int = 0
     row_expr: Optional[IExpr] = None
     name: str = ""
+    replicated: bool = False  # a two-stage model's pattern over columns replicated per scenario
 
 
 @dataclass
@@ -577,7 +578,9 @@ class TwoStageModel(Model):
         the same arrays then share columns, so the library evaluates them in one fused group (shared
         loads, sin/cos and Hessian sums) and stores each column once.  1000 buses x 256 scenarios: the
         five branch-flow patterns had exceeded a group's 16 columns; constraints, Jacobian CSC and
-        Hessian CSC took 469 us together, now 239 us."""
+        Hessian CSC took 469 us together, now 239 us.  FP64 only: a mixed-precision model gets a copy
+        per pattern at creation, because fused patterns share FP32 subexpressions and so round
+        differently from the same patterns each over columns of its own."""
         key = (kind, content)
         if key not in self._columns:
             self._columns[key] = make()
@@ -587,7 +590,7 @@ class TwoStageModel(Model):
         if not scenario:
             return super().add_obj(fn, data, n, name)
         rep, n = self._replicate(data, n)
-        return super().add_obj(fn, rep, n * self.nscen, name)
+        return self._mark(super().add_obj(fn, rep, n * self.nscen, name))
 
     def add_con(self, fn, data=None, n=None, name: str = "", scenario: bool = False) -> ConBlock:
         if not scenario:
@@ -596,6 +599,7 @@ class TwoStageModel(Model):
             return blk
         rep, n = self._replicate(data, n)
         blk = super().add_con(fn, rep, n * self.nscen, name)
+        self._mark(blk.pattern_index)
         for s in range(self.nscen):
             self._cstage.append((blk.row_base + s * n, n, s + 1))
         return ScenarioConBlock(blk.row_base, blk.n_rows, blk.pattern_index, n_per=n)
@@ -613,7 +617,11 @@ class TwoStageModel(Model):
         def shifted(d):
             idx, val = fn(d)
             return _ilift(idx) + d.s * block.n_per, val
-        return super().add_con_aug(block, shifted, rep, n * self.nscen, name)
+        return self._mark(super().add_con_aug(block, shifted, rep, n * self.nscen, name))
+
+    def _mark(self, pattern: int) -> int:
+        self.patterns[pattern].replicated = True
+        return pattern
 
     def var_stage(self) -> np.ndarray:
         out = np.zeros(self.nvar, dtype=np.int32)
@@ -653,6 +661,7 @@ class FlatPattern:
     ftype: np.ndarray
     fields: List[np.ndarray]
     name: str = ""
+    replicated: bool = False  # columns may be one array with other patterns' (see TwoStageModel)
 
 
 @dataclass
@@ -724,4 +733,4 @@ def flatten_pattern(p: Pattern) -> FlatPattern:
         np.array(vop, np.int32), np.array(va, np.int32), np.array(vb, np.int32),
         np.array(vi, np.int64), np.array(vf, np.float64),
         np.array(iop, np.int32), np.array(ia, np.int32), np.array(ib, np.int32),
-        np.array(ii, np.int64), ftype, list(p.fields), p.name)
+        np.array(ii, np.int64), ftype, list(p.fields), p.name, p.replicated)

@@ -328,8 +328,9 @@ exa_status exa_eval_all_host(exa_model *m, const double *x, const double *y, dou
                              double *jac_csc, double *hess_csc);
 
 /* Products at x (NLPModels jprod!/jtprod!/hprod!): Jv[ncon] = J(x) v, Jtw[nvar] = J(x)^T w,
- * Hv[nvar] = (sigma Hess f + sum y_r Hess c_r)(x) v with the Hessian's full symmetric action.  Matrix-free:
- * derivatives are contracted with the vector where they are formed. */
+ * Hv[nvar] = (sigma Hess f + sum y_r Hess c_r)(x) v with the Hessian's full symmetric action.  FP64:
+ * matrix-free, derivatives are contracted with the vector where they are formed.  Mixed precision: the
+ * products of the entries that exa_jac_coord and exa_hess_csc return. */
 exa_status exa_jprod(exa_model *m, const double *x, const double *v, double *Jv);
 exa_status exa_jtprod(exa_model *m, const double *x, const double *w, double *Jtw);
 exa_status exa_hprod(exa_model *m, const double *x, const double *y, double sigma,
@@ -367,7 +368,8 @@ exa_status exa_compile_check(const exa_model_desc *desc, const exa_options *opt,
  * chunk's); waits for the call's end;
  * -1 when no call has recorded them.  "eval_kernel_kind": the generated kernel(s) an exa_eval_all
  * call with every output runs: 0 exa_all, 1 exa_all_b (COO and compressed Hessian sums),
- * 2 exa_first + exa_hess, 3 exa_first + exa_hess_b.
+ * 2 exa_first + exa_hess, 3 exa_first + exa_hess_b.  "hprod_route": exa_hprod adds up 0 per-instance terms,
+ * 1 the Hessian's CSC values, one lane per variable, 2 the same, long rows split.
  * Unknown key: EXA_E_INVALID. */
 exa_status exa_stat(const exa_model *m, const char *key, double *value);
 

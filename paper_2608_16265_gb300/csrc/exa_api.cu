@@ -38,7 +38,7 @@ typedef long long i64;
 // ------------------------------------------------------------------ static kernels
 namespace {
 
-// Hv[i] from the lower-triangle CSC values (hprod_csc): column i holds (r, i), r >= i, giving H_ir v_r; the
+// Hv[i] from the lower-triangle CSC values (HPROD_LANE): column i holds (r, i), r >= i, giving H_ir v_r; the
 // row-sorted permutation lists the entries (i, c), c < i, giving H_ic v_c.
 __global__ void k_hprod_csc(const int *__restrict__ colptr, const int *__restrict__ rowval,
                             const double *__restrict__ val, const int *__restrict__ rptr,
@@ -53,6 +53,17 @@ __global__ void k_hprod_csc(const int *__restrict__ colptr, const int *__restric
         if (c != i) s += val[p] * v[c];
     }
     out[i] = s;
+}
+
+// the variables that the 2 n terms of H v from n CSC entries are added to :
+// term p < n is entry p times v at its row, for its column; term n + p the entry times v at its column, for
+// its row, or for nobody (key nvar) when that is its column
+__global__ void k_sym_keys(const int *__restrict__ row, const int *__restrict__ col, unsigned long long *keys, int n,
+                           int nvar) {
+    int p = blockIdx.x * blockDim.x + threadIdx.x;
+    if (p >= n) return;
+    keys[p] = (unsigned)col[p];
+    keys[(i64)n + p] = (unsigned)(row[p] == col[p] ? nvar : row[p]);
 }
 
 // colof[p] = column of CSC position p
@@ -314,7 +325,13 @@ struct exa_model {
     i64 nnzt = 0, nnzu = 0;
     int *d_tvar = nullptr, *d_uvar = nullptr;
     double *d_prod = nullptr;
-    bool hprod_csc = false;  // H v from the CSC values: few entries, or more terms than 32-bit indices reach
+    // Mixed precision: J v (sum_r, by row) and J^T w (sum_t) from the COO values of the Jacobian's own
+    // kernel, so that the products are those of its FP32-rounded entries
+    GatherSum sum_r;
+    // H v: per-instance terms (FP64), one lane per variable over the CSC values, or sums by length over
+    // the CSC values (sum_u)
+    enum { HPROD_TERMS, HPROD_LANE, HPROD_ENTRIES } hprod_how = HPROD_TERMS;
+    int *d_hother = nullptr;  // HPROD_ENTRIES: the variable that each term's entry is multiplied with
     // Member-chunked exa_eval_all: the members are split into nchunks contiguous groups; the
     // evaluation of group c + 1 runs on the model stream while the reductions of group c run on a
     // side stream.  Per member b (nb + 1 boundaries each): first tile of every kernel kind, and the
@@ -346,7 +363,7 @@ struct exa_model {
     bool use_hcomp = false;       // ... and feed the Hessian CSC (tuner choice)
     int *d_hcrow = nullptr, *d_hccol = nullptr, *d_hcperm = nullptr, *d_hcsegptr = nullptr;
     double *d_hcbuf = nullptr;
-    // Hessian CSC seen by rows (hprod_csc): column of each CSC entry, row-sorted permutation
+    // Hessian CSC seen by rows (HPROD_LANE): column of each CSC entry, row-sorted permutation
     int *d_hcolof = nullptr, *d_hcsr_perm = nullptr, *d_hcsr_ptr = nullptr;
     double *d_hcscbuf = nullptr;
     // gradient and augmentation segments
@@ -714,6 +731,12 @@ class Reduction {
         if (n > 0) push(J, j);
         else zero = f;
     }
+    // entry e of the sums' sources stands for its product with vec[other[e]] (exa_red::Jobs)
+    void weigh(const double *vec, const int *other, int wrap = INT32_MAX) {
+        J.vec = vec;
+        J.other = other;
+        J.wrap = wrap;
+    }
     double *zero = nullptr;  // an objective without partials
     bool empty() const { return !J.nj; }
     void stamp(unsigned long long *t) { J.stamp = t; }
@@ -756,7 +779,8 @@ class Reduction {
                 }
             js->every = blocks >= 8192 && js->sums ? (int)(blocks / js->sums) : 1;
             void *args[] = {js};
-            CR(launch_kernel((const void *)exa_red::k_reduce, (unsigned)blocks, exa_red::THREADS, 0, args, st, overlap));
+            const void *fn = js->vec ? (const void *)exa_red::k_reduce<true> : (const void *)exa_red::k_reduce<false>;
+            CR(launch_kernel(fn, (unsigned)blocks, exa_red::THREADS, 0, args, st, overlap));
         }
         return EXA_OK;
     }
@@ -874,6 +898,20 @@ exa_status build_seg_list(exa_model *m, Scratch &S, const int *ptr, const int *p
     return EXA_OK;
 }
 
+// *len = the longest of n segments.
+exa_status longest_segment(exa_model *m, Scratch &S, const int *ptr, int n, int *len) {
+    int *d = nullptr;
+    CR(S.get(&d, 1));
+    CR(cudaMemsetAsync(d, 0, sizeof(int), m->stream));
+    if (n > 0) {
+        k_seg_longest<<<grid_of(n, 256), 256, 0, m->stream>>>(ptr, n, d);
+        CR(cudaGetLastError());
+    }
+    CR(cudaMemcpyAsync(len, d, sizeof(int), cudaMemcpyDeviceToHost, m->stream));
+    CR(cudaStreamSynchronize(m->stream));
+    return EXA_OK;
+}
+
 // The gather-sum over n segments (ptr, perm).  dense: element s is segment s and one-entry (and
 // empty) segments go to the codes; otherwise segment s is summed into element rows[s].  Elements in
 // `skip` are left to somebody else.
@@ -887,13 +925,8 @@ exa_status build_gather_sum(exa_model *m, Scratch &S, const int *ptr, const int 
         CR(cudaGetLastError());
     }
     const int lo = dense ? 1 : 0;
-    int *d_longest = nullptr, longest = 0;
-    CR(S.get(&d_longest, 1));
-    CR(cudaMemsetAsync(d_longest, 0, sizeof(int), m->stream));
-    k_seg_longest<<<grid_of(n, 256), 256, 0, m->stream>>>(ptr, n, d_longest);
-    CR(cudaGetLastError());
-    CR(cudaMemcpyAsync(&longest, d_longest, sizeof(int), cudaMemcpyDeviceToHost, m->stream));
-    CR(cudaStreamSynchronize(m->stream));
+    int longest = 0;
+    if (exa_status e = longest_segment(m, S, ptr, n, &longest)) return e;
     gs->longest = longest;
     if (longest <= lo) return EXA_OK;
     if (longest <= exa_red::SHORT_MAX || ordered) {
@@ -999,6 +1032,9 @@ void set_chunks(exa_model *m, int n) {
     m->chunk_b.push_back(nb);
 }
 
+// H v over the CSC values: the longest row or column that one lane walks.
+constexpr int HPROD_LANE_MAX = 256;
+
 // Per-model structure: CSC of J and H, row groupings, gradient and augmentation segments.
 exa_status build_structure(exa_model *m) {
     Scratch S{m};
@@ -1028,6 +1064,11 @@ exa_status build_structure(exa_model *m) {
         CR(cudaGetLastError());
     }
     if (exa_status e = build_ptr(m, segkey, 32, nseg, m->nvar, &m->d_jcolptr)) return e;
+    if (m->precision != EXA_FP64) {  // J^T w: all entries by column
+        int *ptr = nullptr;
+        if (exa_status e = build_ptr(m, skeys, 32, nj, m->nvar, &ptr)) return e;
+        if (exa_status e = build_gather_sum(m, S, ptr, m->d_jperm, nullptr, (int)m->nvar, true, false, &m->sum_t)) return e;
+    }
     // ---- Hessian CSC
     CR(dalloc(m, &m->d_hperm, nh));
     CR(dalloc(m, &m->d_hcoo2csc, nh));
@@ -1067,33 +1108,14 @@ exa_status build_structure(exa_model *m) {
         CR(dalloc(m, &m->d_hcbuf, nc));
     }
 
-    // H v through the CSC values where the terms outnumber the Hessian's entries by far (patterns over
-    // many variables that their neighbours share) and no entry is a long sum: 100,000 instances of 28
-    // variables, 2.8 M terms and 0.2 M entries, 57 us from the terms, 47 us this way; a network has fewer
-    // terms than entries.
+    // ---- H v.  Per-instance terms, or the CSC values: where the terms outnumber the Hessian's entries by far
+    // (patterns over many variables that their neighbours share) and no entry is a long sum: 100,000
+    // instances of 28 variables, 2.8 M terms and 0.2 M entries, 57 us from the terms, 47 us this way; a
+    // network has fewer terms than entries.  And in mixed precision, whose Hessian is that of its own kernel.
     const GatherSum &hs = m->has_hcomp ? m->sum_hc : m->sum_h;
-    if (m->nnzu > 4 * m->nnzh_csc && hs.longest <= 256) m->hprod_csc = true;
-    // ---- product terms by variable
-    for (int i = 0; i < 2; i++) {
-        const int n = (int)(i ? m->nnzu : m->nnzt);
-        if (i && m->hprod_csc) continue;
-        unsigned long long *pk = nullptr;
-        int *perm = nullptr, *ptr = nullptr;
-        CR(S.get(&pk, n));
-        CR(dalloc(m, &perm, n));
-        if (n) {
-            k_keys1<<<grid_of(n, 256), 256, 0, m->stream>>>(i ? m->d_uvar : m->d_tvar, pk, n);
-            CR(cudaGetLastError());
-        }
-        if (exa_status e = sort_with_perm(m, S, pk, n, bits_of(m->nvar), &skeys, perm)) return e;
-        if (exa_status e = build_ptr(m, skeys, 0, n, m->nvar, &ptr)) return e;
-        if (exa_status e = build_gather_sum(m, S, ptr, perm, nullptr, (int)m->nvar, true, false, i ? &m->sum_u : &m->sum_t))
-            return e;
-    }
-
-    // ---- Hessian CSC by rows
-    if (m->hprod_csc) {
-        const int nc = (int)m->nnzh_csc;
+    const int nc = (int)m->nnzh_csc;
+    if (m->precision != EXA_FP64 || !m->d_uvar || (m->nnzu > 4 * m->nnzh_csc && hs.longest <= 256)) {
+        // Hessian CSC by rows
         CR(dalloc(m, &m->d_hcolof, nc));
         CR(dalloc(m, &m->d_hcsr_perm, nc));
         CR(dalloc(m, &m->d_hcscbuf, nc));
@@ -1107,6 +1129,59 @@ exa_status build_structure(exa_model *m) {
         }
         if (exa_status e = sort_with_perm(m, S, keys, nc, 32 + bits_of(m->nvar), &skeys, m->d_hcsr_perm)) return e;
         if (exa_status e = build_ptr(m, skeys, 32, nc, m->nvar, &m->d_hcsr_ptr)) return e;
+        // one lane per variable for short rows and columns; else sums by length (2 nc terms, 32-bit indices)
+        int longest = 0;
+        for (const int *ptr : {m->d_hcolptr, m->d_hcsr_ptr}) {
+            int n = 0;
+            if (exa_status e = longest_segment(m, S, ptr, (int)m->nvar, &n)) return e;
+            longest = std::max(longest, n);
+        }
+        m->hprod_how = m->precision == EXA_FP64 || longest <= HPROD_LANE_MAX || 2 * (i64)nc >= INT32_MAX ? exa_model::HPROD_LANE
+                                                                                 : exa_model::HPROD_ENTRIES;
+    }
+    // ---- product terms by variable (FP64)
+    for (int i = 0; i < 2; i++) {
+        const int n = (int)(i ? m->nnzu : m->nnzt);
+        if (m->precision != EXA_FP64 || (i && m->hprod_how != exa_model::HPROD_TERMS)) continue;
+        unsigned long long *pk = nullptr;
+        int *perm = nullptr, *ptr = nullptr;
+        CR(S.get(&pk, n));
+        CR(dalloc(m, &perm, n));
+        if (n) {
+            k_keys1<<<grid_of(n, 256), 256, 0, m->stream>>>(i ? m->d_uvar : m->d_tvar, pk, n);
+            CR(cudaGetLastError());
+        }
+        if (exa_status e = sort_with_perm(m, S, pk, n, bits_of(m->nvar), &skeys, perm)) return e;
+        if (exa_status e = build_ptr(m, skeys, 0, n, m->nvar, &ptr)) return e;
+        if (exa_status e = build_gather_sum(m, S, ptr, perm, nullptr, (int)m->nvar, true, false, i ? &m->sum_u : &m->sum_t))
+            return e;
+    }
+    // ---- Jacobian entries by row (mixed; those by column follow the Jacobian CSC above)
+    if (m->precision != EXA_FP64) {
+        int *perm = nullptr, *ptr = nullptr;
+        CR(dalloc(m, &perm, nj));
+        if (nj) {
+            k_keys1<<<grid_of(nj, 256), 256, 0, m->stream>>>(m->d_jrow, keys, nj);
+            CR(cudaGetLastError());
+        }
+        if (exa_status e = sort_with_perm(m, S, keys, nj, bits_of(m->ncon), &skeys, perm)) return e;
+        if (exa_status e = build_ptr(m, skeys, 0, nj, m->ncon, &ptr)) return e;
+        if (exa_status e = build_gather_sum(m, S, ptr, perm, nullptr, (int)m->ncon, true, false, &m->sum_r)) return e;
+    }
+    // ---- both mentions of every Hessian entry by variable
+    if (m->hprod_how == exa_model::HPROD_ENTRIES) {
+        unsigned long long *pk = nullptr;
+        int *perm = nullptr, *ptr = nullptr;
+        CR(S.get(&pk, 2 * (i64)nc));
+        CR(dalloc(m, &perm, 2 * (i64)nc));
+        CR(dalloc(m, &m->d_hother, 2 * (i64)nc));
+        k_sym_keys<<<grid_of(nc, 256), 256, 0, m->stream>>>(m->d_hrowval, m->d_hcolof, pk, nc, (int)m->nvar);
+        CR(cudaGetLastError());
+        CR(cudaMemcpyAsync(m->d_hother, m->d_hrowval, sizeof(int) * nc, cudaMemcpyDeviceToDevice, m->stream));
+        CR(cudaMemcpyAsync(m->d_hother + nc, m->d_hcolof, sizeof(int) * nc, cudaMemcpyDeviceToDevice, m->stream));
+        if (exa_status e = sort_with_perm(m, S, pk, 2 * nc, bits_of(m->nvar + 1), &skeys, perm)) return e;
+        if (exa_status e = build_ptr(m, skeys, 0, 2 * nc, m->nvar, &ptr)) return e;
+        if (exa_status e = build_gather_sum(m, S, ptr, perm, nullptr, (int)m->nvar, true, false, &m->sum_u)) return e;
     }
 
     // ---- gradient segments by variable
@@ -1272,8 +1347,8 @@ exa_status setup_kernels(exa_model *m, int block, int min_blocks = 0) {
     std::string gerr;
     std::string src = exa::generate_source(m->pats, m->groups, cg, &gerr, m->dsmem);
     if (!gerr.empty()) return fail(m, EXA_E_INTERNAL, gerr);
-    std::string psrc;  // the product kernels, once per model
-    if (!m->lib_prod) {
+    std::string psrc;  // the product kernels, once per FP64 model
+    if (!m->lib_prod && m->precision == EXA_FP64) {
         {
             std::lock_guard<std::mutex> lk(g_cubin_mu);
             auto it = g_prod_src.find(src);
@@ -1294,7 +1369,7 @@ exa_status setup_kernels(exa_model *m, int block, int min_blocks = 0) {
         cudaLibraryUnload(m->lib);
         m->lib = nullptr;
     }
-    const bool products = !m->lib_prod;
+    const bool products = !psrc.empty();
     if (exa_status e = compile(m, src, products ? &psrc : nullptr)) return e;
     const int ng = (int)m->groups.size(), nb = m->nb;
     for (int k = 0; k < exa::M_COUNT; k++) {
@@ -1981,9 +2056,11 @@ exa_status create_impl(const exa_model_desc *const *descs, int nb, const exa_opt
             pm.hcbase = m->nnzhc;
             m->nnzhc += pm.n_inst * (i64)G.hc.size();
             pm.tbase = m->nnzt;
-            m->nnzt += pm.n_inst * (i64)G.tsym.size();
             pm.ubase = m->nnzu;
-            m->nnzu += pm.n_inst * (i64)G.usym.size();
+            if (m->precision == EXA_FP64) {
+                m->nnzt += pm.n_inst * (i64)G.tsym.size();
+                m->nnzu += pm.n_inst * (i64)G.usym.size();
+            }
             for (size_t pos = 0; pos < G.pats.size(); pos++) {
                 const int p = G.pats[pos];
                 const exa::Pattern &P = m->pats[p];
@@ -2046,9 +2123,8 @@ exa_status create_impl(const exa_model_desc *const *descs, int nb, const exa_opt
     CR(dalloc(m, &m->d_hcol, m->nnzh));
     CR(dalloc(m, &m->d_gvar, m->nnzg));
     CR(dalloc(m, &m->d_arow, m->naug));
-    m->hprod_csc = m->nnzu >= (1LL << 31);
     CR(dalloc(m, &m->d_tvar, m->nnzt));
-    if (!m->hprod_csc) CR(dalloc(m, &m->d_uvar, m->nnzu));
+    if (m->nnzu < (1LL << 31)) CR(dalloc(m, &m->d_uvar, m->nnzu));
     m->has_hcomp = m->nnzhc < m->nnzh;
     m->use_hcomp = m->has_hcomp && !(o.flags & EXA_FLAG_NO_HCOMP);
     if (m->has_hcomp) {
@@ -2083,7 +2159,7 @@ exa_status create_impl(const exa_model_desc *const *descs, int nb, const exa_opt
     CR(dalloc(m, &m->d_gbuf, m->nnzg));
     CR(dalloc(m, &m->d_abuf, m->naug));
     CR(dalloc(m, &m->d_cbuf, m->ncon));
-    CR(dalloc(m, &m->d_prod, std::max(m->nnzt, m->hprod_csc ? 0 : m->nnzu)));
+    CR(dalloc(m, &m->d_prod, std::max(m->nnzt, m->hprod_how == exa_model::HPROD_TERMS ? m->nnzu : 0)));
     {  // objective partials: one per CTA, at most one per tile; sized for 32-instance tiles
         i64 maxt = 1;
         for (const ExaPM &pm : m->h_pms) maxt += (pm.n_inst + 31) / 32;
@@ -2912,10 +2988,26 @@ exa_status exa_eval_all_host(exa_model *m, const double *x, const double *y, dou
 // values stored, then gathered per row, column and CSC entry): 30,000-bus network 107 -> 45 us, 32
 // networks (15.7 M entries) 313 -> 147 us, 100,000-step rocket 67.8 ms -> 129 us (one variable in
 // every row: its 300,000 terms were added by one lane).
+//
+// Mixed precision multiplies the entries that its Jacobian and Hessian kernels round to FP32 instead
+// (kernels that contract them as they form them let the compiler fuse other FP32 multiplies and adds, and
+// round differently): the values are stored, then multiplied and summed by k_reduce<true>.
+static exa_status reduce_jac(exa_model *m, const GatherSum &gs, const double *x, const double *vec, const int *other,
+                             double *out) {
+    ExaOut o{};
+    o.jac = m->d_jbuf;
+    if (exa_status e = launch_eval(m, exa::M_JAC, x, nullptr, 0.0, o, 0, -1, true)) return e;
+    Reduction r;
+    r.add(gs, m->d_jbuf, out);
+    r.weigh(vec, other);
+    return r.launch(m, m->stream, true);
+}
+
 exa_status exa_jprod(exa_model *m, const double *x, const double *v, double *Jv) {
     if (exa_status e = check_model(m)) return e;
     if (!m->ncon) return EXA_OK;
     CHECK_PTRS(x, v, Jv);
+    if (m->precision != EXA_FP64) return reduce_jac(m, m->sum_r, x, v, m->d_jcol, Jv);
     ExaOut o{};
     o.v = v;
     o.c = Jv;
@@ -2931,6 +3023,7 @@ exa_status exa_jtprod(exa_model *m, const double *x, const double *w, double *Jt
     if (!m->nvar) return EXA_OK;
     CHECK_PTRS(x, Jtw);
     if (m->ncon && !w) return fail(m, EXA_E_INVALID, "NULL w");
+    if (m->precision != EXA_FP64) return reduce_jac(m, m->sum_t, x, w, m->d_jrow, Jtw);
     ExaOut o{};
     o.v = w;
     o.prod = m->d_prod;
@@ -2943,8 +3036,15 @@ exa_status exa_hprod(exa_model *m, const double *x, const double *y, double sigm
     if (!m->nvar) return EXA_OK;
     CHECK_PTRS(x, v, Hv);
     if (m->ncon && !y) return fail(m, EXA_E_INVALID, "NULL y");
-    if (m->hprod_csc) {
-        if (exa_status e = exa_hess_csc(m, x, y, sigma, m->d_hcscbuf)) return e;
+    if (m->hprod_how != exa_model::HPROD_TERMS) {
+        if (m->nnzh)
+            if (exa_status e = exa_hess_csc(m, x, y, sigma, m->d_hcscbuf)) return e;
+        if (m->hprod_how == exa_model::HPROD_ENTRIES) {
+            Reduction r;
+            r.add(m->sum_u, m->d_hcscbuf, Hv);
+            r.weigh(v, m->d_hother, (int)m->nnzh_csc);
+            return r.launch(m, m->stream, true);
+        }
         k_hprod_csc<<<grid_of(m->nvar, 256), 256, 0, m->stream>>>(m->d_hcolptr, m->d_hrowval, m->d_hcscbuf, m->d_hcsr_ptr,
                                                                    m->d_hcsr_perm, m->d_hcolof, v, Hv, (int)m->nvar);
         CR(cudaGetLastError());
@@ -3003,12 +3103,13 @@ exa_status exa_compile_check(const exa_model_desc *desc, const exa_options *opt,
             std::string src = exa::generate_source(tmp.pats, tmp.groups, cg, &gerr);
             if (!gerr.empty()) s = fail(&tmp, EXA_E_INTERNAL, gerr);
             else {
+                const bool products = cg.precision == EXA_FP64;
                 cg.block = PROD_BLOCK;
                 cg.products = true;
-                const std::string psrc = exa::generate_source(tmp.pats, tmp.groups, cg, &gerr);
+                const std::string psrc = products ? exa::generate_source(tmp.pats, tmp.groups, cg, &gerr) : "";
                 dump_source(src + psrc);
                 std::shared_ptr<std::vector<char>> cubin, pcubin;
-                s = cubins_of(&tmp, src, &psrc, &cubin, &pcubin);
+                s = cubins_of(&tmp, src, products ? &psrc : nullptr, &cubin, &pcubin);
             }
         }
     }
@@ -3041,6 +3142,7 @@ exa_status exa_stat(const exa_model *m, const char *key, double *value) {
     else if (k == "eval_lazy") *value = m->lazy_loads;
     else if (k == "eval_stage") *value = m->stage;
     else if (k == "eval_fused_step") *value = m->fused_step;
+    else if (k == "hprod_route") *value = m->hprod_how;
     else if (k == "eval_kernel_ms") {  // evaluation kernel(s) of the latest exa_eval_all step
         float ms = -1.0f;
         unsigned long long t[2];

@@ -799,8 +799,8 @@ static void build_graph(const Pattern &p, const InputMap &im, Graph &g, PatternG
 // reverse pass over all patterns, H v as the forward derivative of that gradient.  The FP64 pipe binds
 // these kernels, so the reverse pass keeps adjoints as sums of products and takes out the factors that
 // all their terms share before it goes on: the flow patterns of a branch, w_p v_f v_t (g_p cos + b_p sin),
-// give v_f v_t (cos (sum w_p g_p) + ...) with two multiply-adds per pattern.  (Mixed precision contracts
-// the FP32-rounded entries themselves, so that its products are those of its Jacobian and Hessian.)
+// give v_f v_t (cos (sum w_p g_p) + ...) with two multiply-adds per pattern.  (Mixed precision multiplies
+// the stored FP32-rounded entries, so that its products are those of its Jacobian and Hessian.)
 struct ProdGraph {
     std::vector<int> jv;      // per position: the row's product (-1: not a constraint)
     std::vector<int> jt, hv;  // per entry of the group's tsym / usym (-1: zero)
@@ -1175,7 +1175,7 @@ struct Emitter {
     const std::vector<PatternGraph> &PG;  // per position in the group
     const CodegenOptions &opt;
     bool warp_sincos = false;         // the function being printed uses exa_sincos64_warp
-    const ProdGraph *prod = nullptr;  // FP64 products (null: contract the derivative entries)
+    const ProdGraph *prod = nullptr;  // FP64 products and compressed sums (null in mixed precision)
     std::ostringstream os;
     std::string pf_text;  // prefetch functions of the last function() (opt.prefetch > 0)
     // shared-memory staging (opt.stage): the last function()'s stage function and its 8- and
@@ -1332,10 +1332,10 @@ struct Emitter {
         const char *W = mixed ? "float" : "double";
         const bool all = mode_all(mode) || mode == M_FIRST;
         const bool hs_coo = mode_hess_coo(mode);
-        const bool hs_comp = (mode_hess_comp(mode) || mode == M_HPROD) && !grp.hc.empty();
+        const bool hs_comp = mode_hess_comp(mode) && !grp.hc.empty();
         const bool jprod = mode == M_JPROD, jtprod = mode == M_JTPROD, hprod = mode == M_HPROD;
         const bool graph_comp = mode == M_HESS_C && prod;
-        const bool graph_prod = (mode_prod(mode) && prod) || graph_comp;
+        const bool graph_prod = mode_prod(mode) || graph_comp;
         const bool want_struct = mode == M_STRUCT;
         // inputs staged in shared memory by the tile loop (s8 / s4: this thread's column of 8- and
         // 4-byte slots of the current buffer, slot j at [j * EXA_BLOCK])
@@ -1600,9 +1600,9 @@ struct Emitter {
                        << "    so.hcol[pm.hbase[" << P << "] + kk * " << p.nh() << " + " << j << "] = (int)(ga > gb ? gb : ga); }\n";
                 }
             }
-            for (size_t q = 0; q < grp.tsym.size(); q++)
+            for (size_t q = 0; q < (mixed ? 0 : grp.tsym.size()); q++)
                 os << "  so.tvar[pm.tbase + " << q << " * pm.n_inst + kk] = (int)(pm.xoff + i" << grp.tsym[q] << ");\n";
-            if (!grp.usym.empty()) {
+            if (!mixed && !grp.usym.empty()) {
                 os << "  if (so.uvar) {\n";
                 for (size_t q = 0; q < grp.usym.size(); q++)
                     os << "    so.uvar[pm.ubase + " << q << " * pm.n_inst + kk] = (int)(pm.xoff + i" << grp.usym[q] << ");\n";
@@ -1850,17 +1850,7 @@ struct Emitter {
             }
             // a block of S slots per instance: stage the warp's 32 x S values, then write the warp's
             // contiguous run of nact x S values with consecutive lanes on consecutive addresses
-            if (jprod) {
-                // the row's product: its derivatives are never stored
-                std::string sum;
-                for (int sy : p.jsym)
-                    sum += (sum.empty() ? "" : " + ") + widen(G.grad[sy]) + " * V" + std::to_string(grp.sym[pos][sy]);
-                if (sum.empty()) sum = "0.0";
-                if (p.kind == EXA_CON) os << "  if (act) o.c[row" << P << "] = " << sum << ";\n";
-                else os << "  if (act) o.abuf[pm.abase[" << P << "] + kk] = " << sum << ";\n";
-            } else if (jtprod) {
-                for (int sy : p.jsym) accumulate(grp.sym[pos][sy], widen(G.grad[sy]) + " * W" + P);
-            } else if (w.grad && p.nj() > 0) {
+            if (w.grad && p.nj() > 0) {
                 std::vector<std::string> vals;
                 for (int j = 0; j < p.nj(); j++) vals.push_back(widen(G.grad[p.jsym[j]]));
                 if (obj) {
@@ -1906,7 +1896,7 @@ struct Emitter {
                     }
                     os << "  double " << hv << " = " << v << ";\n";
                     vals.push_back(hv);
-                    if (a != b && !hprod) {
+                    if (a != b) {
                         const int ga = grp.sym[pos][a], gb = grp.sym[pos][b];
                         const std::string c =
                             use_eqm ? "((eqm >> " + std::to_string(eqbit.at({std::min(ga, gb), std::max(ga, gb)})) + ") & 1ull)"
@@ -1959,22 +1949,12 @@ struct Emitter {
                     os << "  double hc" << c << " = " << (hc_dsign[c] < 0 ? "exa_neg(" + src + ")" : src) << ";\n";
                     hc_started[c] = 1;
                 }
-            // H v: an entry over two symbols contributes to both, so that two symbols that resolve to one
-            // variable need no doubling
-            if (hprod)
-                for (size_t c = 0; c < grp.hc.size(); c++) {
-                    if (!hc_started[c]) continue;
-                    const int ga = grp.hc_sym[c].first, gb = grp.hc_sym[c].second;
-                    const std::string h = "hc" + std::to_string(c);
-                    accumulate(ga, h + " * V" + std::to_string(gb));
-                    if (ga != gb) accumulate(gb, h + " * V" + std::to_string(ga));
-                }
             // sums over two different symbols that resolve to one variable: doubled as a whole
             std::string any;
             std::vector<std::pair<size_t, std::string>> dbl;
             for (size_t c = 0; c < grp.hc.size(); c++) {
                 const int ga = grp.hc_sym[c].first, gb = grp.hc_sym[c].second;
-                if (!hc_started[c] || ga == gb || hprod) continue;
+                if (!hc_started[c] || ga == gb) continue;
                 auto eb = eqbit.find({std::min(ga, gb), std::max(ga, gb)});
                 const std::string cond = use_eqm && eb != eqbit.end()
                                              ? "((eqm >> " + std::to_string(eb->second) + ") & 1ull)"
@@ -1987,15 +1967,13 @@ struct Emitter {
                 for (auto &d : dbl) os << "    if (" << d.second << ") hc" << d.first << " += hc" << d.first << ";\n";
                 os << "  }\n";
             }
-            if (!hprod) {
-                std::vector<std::string> sums;
-                for (size_t c = 0; c < grp.hc.size(); c++) {
-                    const std::string v = hc_started[c] ? "hc" + std::to_string(c) : "0.0";
-                    if (grp.hc_at[c] >= 0) sums.push_back(v);
-                    else os << "  if (act && o.hcomp) o.hcomp[" << hc_slot(c) << "] = " << v << ";\n";
-                }
-                if (!sums.empty()) staged("o.hcomp", "pm.hcbase", grp.hc_rows, sums, nullptr, nullptr);
+            std::vector<std::string> sums;
+            for (size_t c = 0; c < grp.hc.size(); c++) {
+                const std::string v = hc_started[c] ? "hc" + std::to_string(c) : "0.0";
+                if (grp.hc_at[c] >= 0) sums.push_back(v);
+                else os << "  if (act && o.hcomp) o.hcomp[" << hc_slot(c) << "] = " << v << ";\n";
             }
+            if (!sums.empty()) staged("o.hcomp", "pm.hcbase", grp.hc_rows, sums, nullptr, nullptr);
         }
         // one array per group symbol: consecutive lanes store to consecutive addresses as they are, and
         // the sums by variable read consecutive values where variables follow the instances

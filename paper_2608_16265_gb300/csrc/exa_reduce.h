@@ -61,6 +61,11 @@ struct Jobs {
     int sums = 0;   // blocks of the sums, which come first in the list; the streaming jobs follow
     unsigned long long *stamp = nullptr;  // if set: device time (ns) at which the inputs were complete
     int every = 1;  // > 1: every `every`-th block of the launch is one of the sums (while they last)
+    // k_reduce<true>, products of stored entries with a vector: entry e stands for src[e] * vec[other[e]];
+    // e >= wrap for src[e - wrap] (the second mention of a symmetric entry)
+    const double *vec = nullptr;
+    const int *other = nullptr;
+    int wrap = 0x7fffffff;
     Job j[MAX_JOBS];
 };
 
@@ -71,10 +76,16 @@ constexpr int SHORT_MAX = 32;    // longest segment a single lane adds up
 // about 1.2 us for 4 entries per thread.  One 2000-entry variable of 2000 took a warp 42 us, a block 8.
 constexpr int WARP_MAX = 256, BLOCK_MAX = 8192;
 
+template <bool PROD>
+static __device__ __forceinline__ double entry(const Jobs &J, const double *src, int e) {
+    if (!PROD) return __ldcg(src + e);
+    return __ldcg(src + (e >= J.wrap ? e - J.wrap : e)) * J.vec[__ldg(J.other + e)];
+}
+
 // PERM: a block covers ILP x 256 consecutive positions; thread t takes positions t, t + 256, ... so
 // that the index loads and the stores stay coalesced, and its ILP gathers are in flight together.
-template <int ILP>
-static __device__ __forceinline__ void perm_job(const Job &j, int blk) {
+template <int ILP, bool PROD>
+static __device__ __forceinline__ void perm_job(const Jobs &J, const Job &j, int blk) {
     const unsigned i0 = (unsigned)blk * (THREADS * ILP) + threadIdx.x;
     const int left = (int)((unsigned)j.n - i0);  // may be negative
     int p[ILP];
@@ -86,7 +97,7 @@ static __device__ __forceinline__ void perm_job(const Job &j, int blk) {
     const double *src = wait_inputs(j.src);
     double v[ILP];
 #pragma unroll
-    for (int u = 0; u < ILP; u++) v[u] = p[u] >= 0 ? __ldcg(src + p[u]) : 0.0;
+    for (int u = 0; u < ILP; u++) v[u] = p[u] >= 0 ? entry<PROD>(J, src, p[u]) : 0.0;
     double *dst = j.dst + i0;
 #pragma unroll
     for (int u = 0; u < ILP; u++)
@@ -97,8 +108,8 @@ static __device__ __forceinline__ void perm_job(const Job &j, int blk) {
 // positions: all lanes gather that range in pieces of 256 into shared memory (8 independent loads
 // per lane), then every lane adds up its own G segments from there.
 constexpr int PIECE = 256;
-template <int G>
-static __device__ __forceinline__ void seg_job(const Job &j, int blk, double *buf) {
+template <int G, bool PROD>
+static __device__ __forceinline__ void seg_job(const Jobs &J, const Job &j, int blk, double *buf) {
     const int lane = threadIdx.x & 31;
     const unsigned s0 = ((unsigned)blk * (THREADS / 32) + (threadIdx.x >> 5)) * (32 * G);
     if (s0 >= (unsigned)j.n) {
@@ -124,7 +135,7 @@ static __device__ __forceinline__ void seg_job(const Job &j, int blk, double *bu
     for (int c0 = beg;;) {
 #pragma unroll
         for (int u = 0; u < PIECE / 32; u++)
-            if (p[u] >= 0) b[lane + 32 * u] = __ldcg(src + p[u]);
+            if (p[u] >= 0) b[lane + 32 * u] = entry<PROD>(J, src, p[u]);
         __syncwarp();
         const int c1 = min(c0 + PIECE, end);
 #pragma unroll
@@ -147,15 +158,16 @@ static __device__ __forceinline__ void seg_job(const Job &j, int blk, double *bu
 
 // Sum over [beg, end) of src[perm[q]] (perm null: src[q]) by `width` threads, this one being number t:
 // strided partial sums with 8 independent gathers in flight per thread.
+template <bool PROD = false>
 static __device__ __forceinline__ double strided_sum(const double *src, const int *perm, int beg, int end, int t,
-                                                     int width) {
+                                                     int width, const Jobs *J = nullptr) {
     double s = 0.0;
     for (unsigned q = beg + t; q < (unsigned)end; q += 8 * width) {  // end < 2^31: no wrap
         double v[8];
 #pragma unroll
         for (int u = 0; u < 8; u++) {
             const unsigned e = q + u * width;
-            v[u] = e < (unsigned)end ? (perm ? src[__ldg(perm + e)] : src[e]) : 0.0;
+            v[u] = e >= (unsigned)end ? 0.0 : PROD ? entry<true>(*J, src, __ldg(perm + e)) : perm ? src[__ldg(perm + e)] : src[e];
         }
 #pragma unroll
         for (int u = 0; u < 8; u++) s += v[u];
@@ -177,6 +189,7 @@ static __device__ __forceinline__ double block_sum(double s, double *buf) {
     return t;
 }
 
+template <bool PROD>
 static __global__ void __launch_bounds__(THREADS, 6) k_reduce(const __grid_constant__ Jobs J) {
     __shared__ double buf[(THREADS / 32) * PIECE];
     if (J.stamp && blockIdx.x == 0 && threadIdx.x == 0) {
@@ -196,19 +209,20 @@ static __global__ void __launch_bounds__(THREADS, 6) k_reduce(const __grid_const
     const int w = threadIdx.x >> 5, lane = threadIdx.x & 31;
     switch (j.kind) {
     case PERM:
-        if (j.wide) perm_job<8>(j, blk);
-        else perm_job<2>(j, blk);
+        if (j.wide) perm_job<8, PROD>(J, j, blk);
+        else perm_job<2, PROD>(J, j, blk);
         break;
     case SEG:
-        if (j.wide) seg_job<2>(j, blk, buf);
-        else seg_job<1>(j, blk, buf);
+        if (j.wide) seg_job<2, PROD>(J, j, blk, buf);
+        else seg_job<1, PROD>(J, j, blk, buf);
         break;
     case WSEG: case CSUM: {
         const int s = blk * (THREADS / 32) + w;
         const double *src = wait_inputs(j.src);
         if (s >= j.n) break;
         const int *r = j.kind == CSUM ? j.ptr + s : j.ptr + 2 * (long long)s;
-        const double t = warp_sum(strided_sum(src, j.kind == CSUM ? nullptr : j.perm, __ldg(r), __ldg(r + 1), lane, 32));
+        // (the pieces of a long segment are sums already: never in a k_reduce<true> launch)
+        const double t = warp_sum(strided_sum<PROD>(src, j.kind == CSUM ? nullptr : j.perm, __ldg(r), __ldg(r + 1), lane, 32, &J));
         if (lane == 0) {
             double *d = j.dst + __ldg(j.row + s);
             *d = j.add ? *d + t : t;
@@ -217,7 +231,7 @@ static __global__ void __launch_bounds__(THREADS, 6) k_reduce(const __grid_const
     }
     case CHUNK: case BSEG: {
         const double *src = wait_inputs(j.src);
-        const double t = block_sum(strided_sum(src, j.perm, __ldg(j.ptr + 2 * (long long)blk), __ldg(j.ptr + 2 * (long long)blk + 1), threadIdx.x, THREADS), buf);
+        const double t = block_sum(strided_sum<PROD>(src, j.perm, __ldg(j.ptr + 2 * (long long)blk), __ldg(j.ptr + 2 * (long long)blk + 1), threadIdx.x, THREADS, &J), buf);
         if (threadIdx.x == 0) {
             double *d = j.dst + (j.kind == BSEG ? __ldg(j.row + blk) : blk);
             *d = j.add ? *d + t : t;

@@ -136,8 +136,8 @@ typedef struct {
     int32_t precision;     /* exa_precision */
     int32_t device;        /* CUDA device ordinal */
     int32_t block_threads; /* threads per CTA of the evaluation kernels (multiple of 32, <= 1024);
-                              0 = chosen by the autotuner among 64 / 128 / 256; 64 for models too
-                              small for it, 128 when tuning is off */
+                              0 = chosen by the autotuner among 64 / 128 / 256; without it 64 for
+                              FP64 models too small for it, 128 otherwise */
     int32_t flags;         /* EXA_FLAG_* */
     int32_t grid_factor;   /* evaluation grid: 0 = chosen by the autotuner (one CTA per tile when
                               tuning is off), -1 = one CTA per tile, n > 0 = persistent grid of n

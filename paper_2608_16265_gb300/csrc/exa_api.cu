@@ -2113,7 +2113,9 @@ exa_status create_impl(const exa_model_desc *const *descs, int nb, const exa_opt
     // CTA: their few instances spread over more SMs, and a step is a chain of latencies.  us per step
     // at 32 / 64 / 128 threads: 1000-variable model 11.2 / 11.2 / 12.1, 500-bus network 17.2 / 15.2 / 15.2,
     // 6000-bus 17.1 / 15.3 / 16.5, 20,000-step rocket 21.6 / 23.1 / 25.7.
-    if (!o.block_threads && tiles_of_128(m) < TUNE_TILES) m->block = 64;
+    // FP64 only: another CTA size lets the compiler fuse other FP32 multiplies and adds, and mixed-precision
+    // results would round differently.
+    if (!o.block_threads && m->precision == EXA_FP64 && tiles_of_128(m) < TUNE_TILES) m->block = 64;
     if (exa_status e = setup_kernels(m, m->block, o.min_blocks)) return e;
 
     // structure pass on the device

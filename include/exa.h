@@ -269,8 +269,8 @@ exa_status exa_obj(exa_model *m, const double *x, double *f);
 exa_status exa_obj_noalloc(exa_model *m, const double *x, double *f);
 
 /* g[nvar] = grad f(x): each objective instance writes its own gradient slots, then a gather
- * segmented sum per variable produces g (Sec. 7.2.3, no atomics); slots that are their variables' only
- * ones are written to g directly. */
+ * segmented sum per variable produces g (Sec. 7.2.3, no atomics); in FP64, slots that are their variables'
+ * only ones are written to g directly. */
 exa_status exa_grad(exa_model *m, const double *x, double *g);
 
 /* c[ncon] = base rows plus augmentation terms (Sec. 3.3, 7.2.3). */

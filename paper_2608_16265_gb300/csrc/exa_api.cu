@@ -1202,12 +1202,12 @@ exa_status build_structure(exa_model *m) {
         CR(cudaGetLastError());
     }
     m->grad_compact = 2 * (i64)nseg < m->nvar;
-    // Patterns all of whose slots are the only ones of their variables write the gradient themselves
+    // FP64: patterns all of whose slots are the only ones of their variables write the gradient themselves
     // (ExaPM::gsole); those variables are left out of the sums.  (The slot buffer and the sum moved 36
-    // bytes per variable: PDE 1000^2 step 78.2 -> 73.9 us, 2001^2 mixed 274 -> 256 us.)
+    // bytes per variable: PDE 1000^2 step 78.2 -> 73.9 us.)
     unsigned *sole = nullptr;  // their bits
     i64 n_sole = 0;
-    if (ng) {
+    if (ng && m->precision == EXA_FP64) {
         std::vector<int> start, shared;
         std::vector<std::pair<size_t, int>> owner;  // (descriptor, position) of every block of slots
         for (size_t i = 0; i < m->h_pms.size(); i++) {

@@ -1406,7 +1406,7 @@ struct Emitter {
         for (int pos : act) {
             const Pattern &p = pat(pos);
             if (want_struct) for (int s = 0; s < p.nsym; s++) idx_syms.insert(grp.sym[pos][s]);
-            if ((jprod || p.kind == EXA_OBJ) && want[pos].grad) for (int s = 0; s < p.nsym; s++) idx_syms.insert(grp.sym[pos][s]);
+            if ((jprod || (p.kind == EXA_OBJ && !mixed)) && want[pos].grad) for (int s = 0; s < p.nsym; s++) idx_syms.insert(grp.sym[pos][s]);
             if (want[pos].hess)
                 for (auto &pr : p.hpair)
                     if (pr.first != pr.second || hprod) { idx_syms.insert(grp.sym[pos][pr.first]); idx_syms.insert(grp.sym[pos][pr.second]); }
@@ -1853,16 +1853,19 @@ struct Emitter {
             if (w.grad && p.nj() > 0) {
                 std::vector<std::string> vals;
                 for (int j = 0; j < p.nj(); j++) vals.push_back(widen(G.grad[p.jsym[j]]));
-                if (obj) {
-                    // slots that are their variables' only ones go to the gradient itself
+                // FP64: slots that are their variables' only ones go to the gradient itself.  (Mixed precision:
+                // no; the branch alone makes the compiler fuse other FP32 multiplies and adds in the whole
+                // kernel, and results round differently.)
+                if (obj && !mixed) {
                     os << "  if (o.g && ((pm.gsole >> " << P << ") & 1u)) {\n";
                     for (int j = 0; j < p.nj(); j++)
                         os << "    if (act) o.g[pm.xoff + i" << grp.sym[pos][p.jsym[j]] << "] = " << vals[j] << ";\n";
                     os << "  } else {\n";
                     staged("o.gbuf", "pm.gbase[" + P + "]", p.nj(), vals, nullptr, nullptr);
                     os << "  }\n";
-                }
-                else staged("o.jac", "pm.jbase[" + P + "]", p.nj(), vals, "o.jcsc", "o.jmap");
+                } else if (obj) {
+                    staged("o.gbuf", "pm.gbase[" + P + "]", p.nj(), vals, nullptr, nullptr);
+                } else staged("o.jac", "pm.jbase[" + P + "]", p.nj(), vals, "o.jcsc", "o.jmap");
             }
             if (w.hess) {
                 os << "  const " << W << " w" << P << " = " << (obj ? (mixed ? "exa_d2f(sigma)" : "sigma")

@@ -603,7 +603,7 @@ exa_status compile(exa_model *m, const std::string &src, const std::string *psrc
     return EXA_OK;
 }
 
-// Programmatic stream serialization (every evaluation and reduction kernel waits for the kernels before
+// Programmatic stream serialization (every reduction kernel and FP64 evaluation kernel waits for the kernels before
 // it with griddepcontrol before it touches their results, so its launch may overlap their end) is
 // used in plain streams and in the library's own graphs.  Inside a capture that the caller makes the
 // launches stay ordinary ones.
@@ -637,7 +637,8 @@ int block_of(const exa_model *m, int mode) { return exa::mode_prod(mode) ? PROD_
 int eval_grid(const exa_model *m, Mode mode, int nt) { return m->grid[mode] > 0 ? std::min(m->grid[mode], nt) : nt; }
 
 // The evaluation kernel of `mode` over its tiles [t0, t1) (t1 < 0: all tiles) on the model stream.
-// overlap: its launch may overlap the end of the kernel before it.
+// overlap: its launch may overlap the end of the kernel before it (FP64; mixed-precision kernels do not
+// wait for the kernels ahead of them).
 exa_status launch_eval(exa_model *m, Mode mode, const double *x, const double *y, double sigma, ExaOut out,
                        int t0 = 0, int t1 = -1, bool overlap = false) {
     if (t1 < 0) t1 = m->ntiles[mode];
@@ -651,7 +652,7 @@ exa_status launch_eval(exa_model *m, Mode mode, const double *x, const double *y
     int pfd = m->pfd[mode];
     void *args[] = {&tiles, &nt, &m->d_pm, &x, &y, &th, &sigma, &out, &so, &pfd};
     CR(launch_kernel((const void *)m->fn[mode], eval_grid(m, mode, nt), block_of(m, mode), (size_t)m->dsmem[mode], args,
-                     m->stream, overlap && may_overlap(m)));
+                     m->stream, overlap && m->precision == EXA_FP64 && may_overlap(m)));
     return EXA_OK;
 }
 

@@ -2307,7 +2307,10 @@ std::string generate_source(const std::vector<Pattern> &pats, const std::vector<
         // has finished its tiles.  (Let in at the start they crowd the SMs that empty first: constraints
         // + Jacobian CSC + Hessian CSC of a 30,000-variable model took 66 us, 40 us without any
         // overlap, 27 us this way; a 30,000-bus network's products 54, 59 and 42 us.)
-        if (m != M_STRUCT)
+        // FP64 only: in mixed precision the wait makes the compiler fuse other FP32 multiplies and adds in
+        // some models (2e-8 of the largest element), for 4 us of a 30,000-bus network's five callbacks
+        // (43 / 47 us) and 7 of the 256-network batch's step (708 / 716 us).
+        if (m != M_STRUCT && !mixed)
             src << "  asm volatile(\"griddepcontrol.wait;\" : \"+l\"(x), \"+l\"(y), \"+l\"(th) : : \"memory\");\n";
         if (mode_all(m) || m == M_FIRST)
             src << "  if (o.stamp && blockIdx.x == 0 && threadIdx.x == 0) asm volatile(\"mov.u64 %0, %%globaltimer;\" : \"=l\"(*o.stamp) : : \"memory\");\n";
@@ -2400,7 +2403,7 @@ std::string generate_source(const std::vector<Pattern> &pats, const std::vector<
         src << "      default: break;\n    }\n  }\n";
         if (stk) src << "  sbuf ^= 1;\n";
         src << "  }\n";
-        if (m != M_STRUCT) src << "  asm volatile(\"griddepcontrol.launch_dependents;\" ::: \"memory\");\n";
+        if (m != M_STRUCT && !mixed) src << "  asm volatile(\"griddepcontrol.launch_dependents;\" ::: \"memory\");\n";
         if (stk) src << "  asm volatile(\"cp.async.wait_group 0;\" ::: \"memory\");  // nothing in flight at exit\n";
         if (objred) {
             // Every thread sums the objective terms of all its instances over the CTA's tiles (in tile

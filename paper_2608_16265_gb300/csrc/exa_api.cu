@@ -1895,7 +1895,7 @@ exa_status build_groups(exa_model *m, const exa_model_desc *const *descs, int nb
         G.nic = (int)A.ics.size();
         G.nfc = (int)A.fcs.size();
     }
-    for (auto &G : m->groups) exa::finalize_group(G, m->pats);
+    for (auto &G : m->groups) exa::finalize_group(G, m->pats, m->precision != EXA_FP64);
     return EXA_OK;
 }
 
@@ -3087,6 +3087,7 @@ exa_status exa_compile_check(const exa_model_desc *desc, const exa_options *opt,
     } else {
         exa_options o{};
         if (opt) o = *opt;
+        tmp.precision = o.precision;
         s = load_patterns(*desc, &tmp);
         const exa_model_desc *d1[1] = {desc};
         if (s == EXA_OK) s = build_groups(&tmp, d1, 1, (o.flags & EXA_FLAG_NO_FUSE) == 0);

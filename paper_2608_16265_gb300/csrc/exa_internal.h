@@ -141,7 +141,7 @@ struct Group {
     std::vector<std::vector<std::pair<int, int>>> hc;
     std::vector<std::pair<int, int>> hc_sym;  // group symbol pair of each compressed slot
     // where a compressed slot lies in the group's part of the buffer: hc_at >= 0: at kk * hc_rows + hc_at
-    // (rows of neighbouring slots per instance); hc_at < 0, both variables follow the instance number:
+    // (rows of neighbouring slots per instance); hc_at < 0, both variables follow the instance number (FP64):
     // array (hc_rows - 1 - hc_at) of n_inst entries, so that the sums by variable read neighbours
     std::vector<int> hc_at;
     int hc_rows = 0;
@@ -150,7 +150,7 @@ struct Group {
 
 // Unifies the symbols of a group's patterns: equal index expressions (columns compared as group
 // columns, member-varying constants as slots) are one group symbol.
-void finalize_group(Group &g, const std::vector<Pattern> &pats);
+void finalize_group(Group &g, const std::vector<Pattern> &pats, bool mixed);
 
 // Validates a pattern (tree shape, opcodes, field types) and computes symbols and slot tables.
 // Returns an empty string on success, else the error message.

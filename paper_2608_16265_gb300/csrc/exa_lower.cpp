@@ -1085,7 +1085,7 @@ static std::string group_idx_key(const Pattern &p, const std::vector<int> &field
     }
 }
 
-void finalize_group(Group &g, const std::vector<Pattern> &pats) {
+void finalize_group(Group &g, const std::vector<Pattern> &pats, bool mixed) {
     std::map<std::string, int> ids;
     g.sym.assign(g.pats.size(), {});
     g.sym_root.clear();
@@ -1117,9 +1117,10 @@ void finalize_group(Group &g, const std::vector<Pattern> &pats) {
         const INode &n = p.ix[r];
         return n.op == EXA_I_FIELD || (n.op >= EXA_I_ADD && (has_field(p, n.a) || has_field(p, n.b)));
     };
-    // (Compressed sums all side by side per instance / like this: 256 networks, every output 794 / 777 us,
-    // mixed 724 / 714 us: the diagonals of the branch flows, a quarter of the sums, are read back in runs
-    // instead of one 32-byte sector each.)
+    // (Compressed sums all side by side per instance / like this: 256 networks, every output 794 / 777 us:
+    // the diagonals of the branch flows, a quarter of the sums, are read back in runs instead of one 32-byte
+    // sector each.  FP64 only: in mixed precision the stores make the compiler fuse other FP32 multiplies and
+    // adds in some models, 6e-9 of the largest element, for 4 us of 720.)
     auto follows = [&](int s) {
         const Pattern &p = pats[g.pats[g.sym_root[s].first]];
         return !has_field(p, g.sym_root[s].second);
@@ -1128,7 +1129,7 @@ void finalize_group(Group &g, const std::vector<Pattern> &pats) {
     g.hc_rows = 0;
     int arrays = 0;
     for (auto &pr : g.hc_sym)
-        g.hc_at.push_back(follows(pr.first) && follows(pr.second) ? -1 - arrays++ : g.hc_rows++);
+        g.hc_at.push_back(!mixed && follows(pr.first) && follows(pr.second) ? -1 - arrays++ : g.hc_rows++);
     std::set<int> t, u;
     for (size_t pos = 0; pos < g.pats.size(); pos++)
         if (pats[g.pats[pos]].kind != EXA_OBJ) t.insert(g.sym[pos].begin(), g.sym[pos].end());

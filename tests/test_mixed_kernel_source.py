@@ -27,3 +27,6 @@ def test_programmatic_launch(generated):
     assert ("griddepcontrol.wait" in src) == fp64 and ("griddepcontrol.launch_dependents" in src) == fp64
 
 
+def test_arrays_of_compressed_sums(generated):
+    fp64, src = generated
+    assert ("if (act && o.hcomp)" in src) == fp64

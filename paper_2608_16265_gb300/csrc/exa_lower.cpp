@@ -812,6 +812,12 @@ class Products {
     std::map<int, bool> dep_;
     std::map<int, int> tan_, leaves_;
     int wrt_ = -1;
+    // Nodes whose derivatives are given: node -> (operand, partial derivative).  The rules of the node's own
+    // operation would be right as well but for rounding: the derivative of u / hypot(u, w) by u comes out as
+    // (1 - (u/v)^2) / v, which has no digits left where w is far below u, and is w^2 / v^3; that of b (u^b / u)
+    // by u has the difference of two nearly equal terms where b is near 1; a power u^-5 as 1 / u^5 overflows in
+    // the square of the quotient where the result does not.
+    std::map<int, std::vector<std::pair<int, int>>> given_;
     typedef std::map<std::vector<int>, double> Terms;  // sorted factors -> coefficient
 
     bool dep(int n) {  // depends on x
@@ -822,6 +828,37 @@ class Products {
         return dep_[n] = d;
     }
     int one() { return g.lit(1.0, PD); }
+    // The derivatives of node n by operands a and b are da and db (negations stripped, as nodes share them).
+    void give(int n, int a, int da, int b, int db) {
+        for (; g.n[n].op == S_NEG; n = g.n[n].a) { da = g.neg(da); db = g.neg(db); }
+        if (g.n[n].op == S_LIT || g.n[n].op == S_IN || given_.count(n)) return;
+        auto &v = given_[n];
+        v.push_back({a, da});
+        if (b >= 0 && b != a) v.push_back({b, db});
+        else if (b >= 0) v[0].second = g.add(da, db);
+    }
+    // Operands of node n that depend on x, with its partial derivatives.
+    std::vector<std::pair<int, int>> partials(int n) {
+        std::vector<std::pair<int, int>> r;
+        auto it = given_.find(n);
+        if (it != given_.end()) {
+            for (auto &p : it->second)
+                if (dep(p.first)) r.push_back(p);
+            return r;
+        }
+        const SN s = g.n[n];
+        for (int which = 0; which < 2; which++) {
+            const int k = which ? s.b : s.a;
+            if (k >= 0 && dep(k)) r.push_back({k, partial(n, which)});
+        }
+        return r;
+    }
+    // First partials d1, d2 of a function of (a, b) with their own derivatives h11, h12, h22.
+    int curved(int which, int a, int b, int d1, int d2, int h11, int h12, int h22) {
+        give(d1, a, h11, b, h12);
+        give(d2, a, h12, b, h22);
+        return which ? d2 : d1;
+    }
     // partial derivatives of node n for its operands, as build_graph forms them
     int partial(int n, int which) {
         const SN s = g.n[n];
@@ -854,17 +891,28 @@ class Products {
         case S_LOG2: case S_LOG10:
             return g.div(one(), g.mul(a, g.lit(s.op == S_LOG2 ? 0.69314718055994531 : 2.3025850929940457, PD)));
         case S_EXP2: return g.mul(n, g.lit(0.69314718055994531, PD));
-        case S_POW: return which ? g.mul(n, g.fn(S_LOG, a)) : g.mul(b, g.div(n, a));
-        case S_ATAN2: {
-            const int r = g.add(g.mul(a, a), g.mul(b, b));
-            return which ? g.neg(g.div(a, r)) : g.div(b, r);
+        case S_POW: {
+            const int la = g.fn(S_LOG, a), q = g.div(n, a);
+            return curved(which, a, b, g.mul(b, q), g.mul(n, la), g.mul(g.mul(b, g.sub(b, one())), g.div(q, a)),
+                          g.mul(q, g.add(one(), g.mul(b, la))), g.mul(n, g.mul(la, la)));
         }
-        case S_HYPOT: return g.div(which ? b : a, n);
+        case S_ATAN2: {
+            const int r = g.add(g.mul(a, a), g.mul(b, b)), r2 = g.mul(r, r);
+            const int ab2 = g.div(g.mul(g.lit(2.0, PD), g.mul(a, b)), r2);
+            return curved(which, a, b, g.div(b, r), g.neg(g.div(a, r)), g.neg(ab2),
+                          g.div(g.sub(g.mul(a, a), g.mul(b, b)), r2), ab2);
+        }
+        case S_HYPOT: {
+            const int n3 = g.mul(n, g.mul(n, n));
+            return curved(which, a, b, g.div(a, n), g.div(b, n), g.div(g.mul(b, b), n3), g.neg(g.div(g.mul(a, b), n3)),
+                          g.div(g.mul(a, a), n3));
+        }
         default: return -1;
         }
     }
     // leaves of node n's product tree (at most 1000)
     int leaves(int n) {
+        if (given_.count(n)) return 1;
         auto it = leaves_.find(n);
         if (it != leaves_.end()) return it->second;
         const SN s = g.n[n];
@@ -876,7 +924,7 @@ class Products {
     void factors(int n, double &c, std::vector<int> &f) {
         const SN s = g.n[n];
         if (s.op == S_NEG) { c = -c; factors(s.a, c, f); }
-        else if (s.op == S_MUL && leaves(n) <= 8) { factors(s.a, c, f); factors(s.b, c, f); }
+        else if (s.op == S_MUL && !given_.count(n) && leaves(n) <= 8) { factors(s.a, c, f); factors(s.b, c, f); }
         else if (s.op == S_LIT) c *= s.lit;
         else f.push_back(n);
     }
@@ -947,19 +995,21 @@ class Products {
             else if (s.iid == wrt_) r[{}] = 1.0;
             return r;
         }
-        for (int which = 0; which < 2; which++) {
-            const int k = which ? s.b : s.a;
-            if (k < 0 || !dep(k)) continue;
-            if (s.op == S_ADD || s.op == S_SUB || s.op == S_NEG) {
+        if (s.op == S_ADD || s.op == S_SUB || s.op == S_NEG) {
+            for (int which = 0; which < 2; which++) {
+                const int k = which ? s.b : s.a;
                 const double sign = s.op == S_NEG || (s.op == S_SUB && which) ? -1.0 : 1.0;
-                for (auto &kv : tangent_terms(k)) r[kv.first] += sign * kv.second;
-            } else {
-                const int d = tangent(k);  // (kept: a square uses its operand's twice)
-                if (d < 0) continue;
+                if (k >= 0)
+                    for (auto &kv : tangent_terms(k)) r[kv.first] += sign * kv.second;
+            }
+        } else {
+            for (auto &p : partials(n)) {
+                const int d = tangent(p.first);  // (kept: a square uses its operand's twice)
+                if (d < 0 || g.zero(p.second)) continue;
                 double c = 1.0;
                 std::vector<int> f;
                 factors(d, c, f);
-                factors(partial(n, which), c, f);
+                factors(p.second, c, f);
                 std::sort(f.begin(), f.end());
                 r[f] += c;
             }
@@ -969,7 +1019,20 @@ class Products {
     }
 
   public:
-    explicit Products(Graph &graph) : g(graph) {}
+    Products(Graph &graph, const std::vector<Pattern> &pats, const Group &grp, const std::vector<PatternGraph> &PG) : g(graph) {
+        for (size_t pos = 0; pos < grp.pats.size(); pos++) {
+            const Pattern &p = pats[grp.pats[pos]];
+            for (size_t i = 0; i < p.v.size(); i++)
+                if (p.v[i].op == EXA_V_POWI && p.v[i].iv < -1) power(PG[pos].val[i], PG[pos].val[p.v[i].a], p.v[i].iv, 2);
+        }
+    }
+    // node n is u^m, m negative: its first `order` derivatives
+    void power(int n, int u, long long m, int order) {
+        if (!order || g.is_lit(u)) return;
+        const int less = g.powi(u, m - 1);
+        give(n, u, g.mul(g.lit((double)m, PD), less), -1, -1);
+        power(less, u, m - 1, order - 1);
+    }
 
     // directions of tangent(): v, or one group symbol
     void direction(int symbol) {
@@ -1005,14 +1068,12 @@ class Products {
             std::vector<int> f;
             collapse(t, c, f);
             if (f.size() > 4) f = {product(f)};
-            for (int which = 0; which < 2; which++) {
-                const int k = which ? s.b : s.a;
-                if (k < 0 || !dep(k)) continue;
+            for (auto &p : partials(n)) {
                 double ck = c;
                 std::vector<int> fk = f;
-                factors(partial(n, which), ck, fk);
+                factors(p.second, ck, fk);
                 std::sort(fk.begin(), fk.end());
-                adj[k][fk] += ck;
+                adj[p.first][fk] += ck;
             }
         }
         return grad;
@@ -1031,7 +1092,7 @@ static std::vector<std::pair<int, int>> curved_values(const std::vector<Pattern>
 static ProdGraph build_products(const std::vector<Pattern> &pats, const Group &grp, Graph &g,
                                 const std::vector<PatternGraph> &PG) {
     ProdGraph r;
-    Products P(g);
+    Products P(g, pats, grp, PG);
     std::vector<std::pair<int, int>> con;
     r.jv.assign(grp.pats.size(), -1);
     for (size_t pos = 0; pos < grp.pats.size(); pos++) {
@@ -1055,7 +1116,7 @@ static ProdGraph build_compressed(const std::vector<Pattern> &pats, const Group 
     ProdGraph r;
     r.hc.assign(grp.hc.size(), -1);
     if (grp.hc.empty()) return r;
-    Products P(g);
+    Products P(g, pats, grp, PG);
     std::map<int, int> gh = P.gradient(curved_values(pats, grp, PG));
     for (int s : grp.usym) {
         P.direction(s);

@@ -403,6 +403,15 @@ cudaError_t dalloc(exa_model *m, T **p, i64 count) {
     }
     return e;
 }
+template <typename T>
+void dfree(exa_model *m, T **p, i64 count) {
+    auto it = std::find(m->allocs.begin(), m->allocs.end(), (void *)*p);
+    if (it == m->allocs.end()) return;
+    m->allocs.erase(it);
+    m->device_bytes -= (size_t)std::max<i64>(count, 1) * sizeof(T);
+    cudaFree(*p);
+    *p = nullptr;
+}
 
 #define CR(call)                                                                                   \
     do {                                                                                           \
@@ -1110,9 +1119,10 @@ exa_status build_structure(exa_model *m) {
     }
 
     // ---- H v.  Per-instance terms, or the CSC values: where the terms outnumber the Hessian's entries by far
-    // (patterns over many variables that their neighbours share) and no entry is a long sum: 100,000
-    // instances of 28 variables, 2.8 M terms and 0.2 M entries, 57 us from the terms, 47 us this way; a
-    // network has fewer terms than entries.  And in mixed precision, whose Hessian is that of its own kernel.
+    // (patterns over many variables that their neighbours share) and no entry is a long sum, no row or column
+    // a long walk: 100,000 instances of 28 variables, 2.8 M terms and 0.2 M entries, 57 us from the terms, 47 us
+    // this way; a network has fewer terms than entries.  And in mixed precision, whose Hessian is that of its
+    // own kernel.
     const GatherSum &hs = m->has_hcomp ? m->sum_hc : m->sum_h;
     const int nc = (int)m->nnzh_csc;
     if (m->precision != EXA_FP64 || !m->d_uvar || (m->nnzu > 4 * m->nnzh_csc && hs.longest <= 256)) {
@@ -1137,8 +1147,15 @@ exa_status build_structure(exa_model *m) {
             if (exa_status e = longest_segment(m, S, ptr, (int)m->nvar, &n)) return e;
             longest = std::max(longest, n);
         }
-        m->hprod_how = m->precision == EXA_FP64 || longest <= HPROD_LANE_MAX || 2 * (i64)nc >= INT32_MAX ? exa_model::HPROD_LANE
-                                                                                 : exa_model::HPROD_ENTRIES;
+        const bool terms = m->precision == EXA_FP64 && m->d_uvar;
+        m->hprod_how = longest <= HPROD_LANE_MAX ? exa_model::HPROD_LANE : terms ? exa_model::HPROD_TERMS
+                       : 2 * (i64)nc < INT32_MAX ? exa_model::HPROD_ENTRIES : exa_model::HPROD_LANE;
+        if (m->hprod_how == exa_model::HPROD_TERMS) {
+            dfree(m, &m->d_hcolof, nc);
+            dfree(m, &m->d_hcsr_perm, nc);
+            dfree(m, &m->d_hcscbuf, nc);
+            dfree(m, &m->d_hcsr_ptr, m->nvar + 1);
+        }
     }
     // ---- product terms by variable (FP64)
     for (int i = 0; i < 2; i++) {

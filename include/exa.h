@@ -270,7 +270,9 @@ exa_status exa_obj_noalloc(exa_model *m, const double *x, double *f);
 
 /* g[nvar] = grad f(x): each objective instance writes its own gradient slots, then a gather
  * segmented sum per variable produces g (Sec. 7.2.3, no atomics); in FP64, slots that are their variables'
- * only ones are written to g directly. */
+ * only ones are written to g directly.
+ * g may be x (the point is then overwritten); as in every call, no other output may overlap an input except
+ * Jv, Jtw and Hv, which may overlap x. */
 exa_status exa_grad(exa_model *m, const double *x, double *g);
 
 /* c[ncon] = base rows plus augmentation terms (Sec. 3.3, 7.2.3). */

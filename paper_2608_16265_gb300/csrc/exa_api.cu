@@ -320,6 +320,7 @@ struct exa_model {
     // Jacobian CSC, Hessian CSC from the COO slots and from the compressed sums, gradient,
     // constraint augmentations
     GatherSum sum_j, sum_h, sum_hc, sum_g, sum_a;
+    GatherSum sum_gall;  // the gradient over every slot, sole ones included (only where there are sole ones)
     // J^T w and H v by variable, from the per-instance terms; work buffer (nnzt / nnzu terms)
     GatherSum sum_t, sum_u;
     i64 nnzt = 0, nnzu = 0;
@@ -1017,6 +1018,7 @@ exa_status build_member_bounds(exa_model *m) {
     if (exa_status e = lists(m->sum_h, as_ll(m->mb_hcsc))) return e;
     if (exa_status e = lists(m->sum_hc, as_ll(m->mb_hcsc))) return e;
     if (exa_status e = lists(m->sum_g, xk)) return e;
+    if (exa_status e = lists(m->sum_gall, xk)) return e;
     if (exa_status e = lists(m->sum_a, ck)) return e;
     m->mb_gseg.assign(nb + 1, 0);
     if (m->n_gseg)
@@ -1263,6 +1265,12 @@ exa_status build_structure(exa_model *m) {
             k_mark_sole<<<grid_of(ng, 256), 256, 0, m->stream>>>(m->d_gvar, ng, d_start, (int)start.size(), d_shared, sole);
             CR(cudaGetLastError());
         }
+    }
+    if (n_sole) {
+        m->sum_gall.sh.n = nseg;
+        m->sum_gall.sh.ptr = m->d_gsegptr;
+        m->sum_gall.sh.perm = m->d_gperm;
+        m->sum_gall.sh.row = m->d_gsegvar;
     }
     if (m->grad_compact) {
         m->sum_g.fill_n = m->nvar;
@@ -2353,16 +2361,38 @@ exa_status exa_obj_noalloc(exa_model *m, const double *x, double *f) {
     return obj_final(m, part, nparts, f, m->stream, true);
 }
 
+static bool overlap(const double *a, i64 na, const double *b, i64 nb) {
+    return a && b && (uintptr_t)a < (uintptr_t)(b + nb) && (uintptr_t)b < (uintptr_t)(a + na);
+}
+
+// A gradient in place of the point (or of y): other instances may still read what a sole slot would
+// overwrite, so every slot goes through the buffer and g is written when the evaluation kernel has ended.
+static bool late_gradient(const exa_model *m, const double *g, const double *x, const double *y) {
+    return m->sum_gall.sh.n && (overlap(g, m->nvar, x, m->nvar) || overlap(g, m->nvar, y, m->ncon));
+}
+
+static const GatherSum &gradient_sums(const exa_model *m, bool late) { return late ? m->sum_gall : m->sum_g; }
+
+// Before a late gradient's sums, which write the variables that have slots: zeros (for members b0 .. b1).
+static exa_status clear_gradient(exa_model *m, double *g, int b0, int b1, cudaStream_t st) {
+    const i64 v0 = m->xoff[b0], v1 = m->xoff[b1];
+    if (v1 > v0) CR(cudaMemsetAsync(g + v0, 0, sizeof(double) * (v1 - v0), st));
+    return EXA_OK;
+}
+
 exa_status exa_grad(exa_model *m, const double *x, double *g) {
     if (exa_status e = check_model(m)) return e;
     CHECK_PTRS(x, g);
+    const bool late = late_gradient(m, g, x, nullptr);
     ExaOut o{};
     o.gbuf = m->d_gbuf;
-    o.g = g;
+    o.g = late ? nullptr : g;
     if (exa_status e = launch_eval(m, exa::M_GRAD, x, nullptr, 0.0, o, 0, -1, true)) return e;
+    if (late)
+        if (exa_status e = clear_gradient(m, g, 0, m->nb, m->stream)) return e;
     Reduction r;
-    r.add(m->sum_g, m->d_gbuf, g);
-    return r.launch(m, m->stream, true);
+    r.add(gradient_sums(m, late), m->d_gbuf, g);
+    return r.launch(m, m->stream, !late);
 }
 
 exa_status exa_cons(exa_model *m, const double *x, double *c) {
@@ -2564,7 +2594,10 @@ static exa_status eval_all_chunked(exa_model *m, const double *x, const double *
         Reduction r;
         if (jside) r.add(m->sum_j, o.jac, jac_csc, false, b0, b1);
         if (hside) r.add(hcomp ? m->sum_hc : m->sum_h, hcomp ? m->d_hcbuf : o.hess, hess_csc, false, b0, b1);
-        if (g) r.add(m->sum_g, m->d_gbuf, g, false, b0, b1);
+        const bool late = g && !o.g;
+        if (late)
+            if (exa_status e = clear_gradient(m, g, b0, b1, ps)) return e;
+        if (g) r.add(gradient_sums(m, late), m->d_gbuf, g, false, b0, b1);
         if (c) r.add(m->sum_a, m->d_abuf, c, true, b0, b1);
         if (exa_status e = r.launch(m, ps, false)) return e;
         if (m->post_chunk)
@@ -2712,7 +2745,8 @@ static exa_status eval_all_launches(exa_model *m, const double *x, const double 
     o.c = c ? c : m->d_cbuf;
     o.abuf = m->d_abuf;
     o.gbuf = m->d_gbuf;
-    o.g = g;
+    const bool late = late_gradient(m, g, x, y);
+    o.g = late ? nullptr : g;
     o.jac = jac ? jac : m->d_jbuf;
     o.hess = hess ? hess : m->d_hbuf;
     // a CSC without duplicates is a permutation of the COO slots: the evaluation kernel writes it
@@ -2755,7 +2789,7 @@ static exa_status eval_all_launches(exa_model *m, const double *x, const double 
     const bool split = want_h && m->split_all;
     Reduction first, second;
     if (f) first.obj(m->d_objpart, eval_grid(m, split ? exa::M_FIRST : mode, m->ntiles[split ? exa::M_FIRST : mode]), f);
-    if (g) first.add(m->sum_g, m->d_gbuf, g);
+    if (g) first.add(gradient_sums(m, late), m->d_gbuf, g);
     if (c) first.add(m->sum_a, m->d_abuf, c, true);
     if (jac_csc && !jdirect) first.add(m->sum_j, o.jac, jac_csc);
     Reduction &hr = split ? second : first;
@@ -2794,12 +2828,14 @@ static exa_status eval_all_launches(exa_model *m, const double *x, const double 
     }
     if (!stamps)
         if (exa_status e = record_eval_event(m, &m->ev_k1, m->stream)) return e;
+    if (split) CR(cudaStreamWaitEvent(m->side, m->ev_first, 0));
+    if (late)
+        if (exa_status e = clear_gradient(m, g, 0, m->nb, split ? m->side : m->stream)) return e;
     if (split) {
-        CR(cudaStreamWaitEvent(m->side, m->ev_first, 0));
         if (exa_status e = first.launch(m, m->side, false)) return e;
         CR(cudaEventRecord(m->ev_join, m->side));
     }
-    if (exa_status e = hr.launch(m, m->stream, true)) return e;
+    if (exa_status e = hr.launch(m, m->stream, split || !late)) return e;
     if (split) CR(cudaStreamWaitEvent(m->stream, m->ev_join, 0));
     return EXA_OK;
 }
@@ -3028,14 +3064,17 @@ exa_status exa_jprod(exa_model *m, const double *x, const double *v, double *Jv)
     if (!m->ncon) return EXA_OK;
     CHECK_PTRS(x, v, Jv);
     if (m->precision != EXA_FP64) return reduce_jac(m, m->sum_r, x, v, m->d_jcol, Jv);
+    double *const out = overlap(Jv, m->ncon, x, m->nvar) ? m->d_cbuf : Jv;  // rows are written while others read x
     ExaOut o{};
     o.v = v;
-    o.c = Jv;
+    o.c = out;
     o.abuf = m->d_abuf;
     if (exa_status e = launch_eval(m, exa::M_JPROD, x, nullptr, 0.0, o, 0, -1, true)) return e;
     Reduction r;
-    r.add(m->sum_a, m->d_abuf, Jv, true);
-    return r.launch(m, m->stream, true);
+    r.add(m->sum_a, m->d_abuf, out, true);
+    if (exa_status e = r.launch(m, m->stream, true)) return e;
+    if (out != Jv) CR(cudaMemcpyAsync(Jv, out, sizeof(double) * m->ncon, cudaMemcpyDeviceToDevice, m->stream));
+    return EXA_OK;
 }
 
 exa_status exa_jtprod(exa_model *m, const double *x, const double *w, double *Jtw) {

@@ -358,6 +358,8 @@ struct exa_model {
     // ... or two device timer stamps, in graphs of one evaluation kernel and its reductions
     unsigned long long *d_stamp = nullptr;
     bool stamped = false;  // the latest call used the stamps
+    cudaEvent_t ev_done = nullptr;            // the latest stamped call's end
+    unsigned long long *h_stamp = nullptr;    // page-locked copy for exa_stat
     bool grad_compact = false;
     int n_gseg = 0;
     int *d_gsegptr = nullptr, *d_gsegvar = nullptr;
@@ -429,7 +431,9 @@ void free_all(exa_model *m) {
     m->cap_stream = nullptr;
     if (m->side) cudaStreamDestroy(m->side);
     m->side = nullptr;
-    for (cudaEvent_t *e : {&m->ev_join, &m->ev_first}) {
+    if (m->h_stamp) cudaFreeHost(m->h_stamp);
+    m->h_stamp = nullptr;
+    for (cudaEvent_t *e : {&m->ev_join, &m->ev_first, &m->ev_done}) {
         if (*e) cudaEventDestroy(*e);
         *e = nullptr;
     }
@@ -2062,6 +2066,8 @@ exa_status create_impl(const exa_model_desc *const *descs, int nb, const exa_opt
     CR(dalloc(m, &m->d_status, 1));
     CR(cudaMemset(m->d_status, 0, sizeof(int)));
     CR(dalloc(m, &m->d_stamp, 2));
+    CR(cudaMallocHost((void **)&m->h_stamp, 2 * sizeof(unsigned long long)));
+    CR(cudaEventCreateWithFlags(&m->ev_done, cudaEventDisableTiming));
     std::vector<ExaPM> pms((size_t)nb * ng);
     for (int b = 0; b < nb; b++) {
         const exa_model_desc &d = *descs[b];
@@ -2840,6 +2846,14 @@ static exa_status eval_all_launches(exa_model *m, const double *x, const double 
     return EXA_OK;
 }
 
+// The graph, and for stamped ones the end that exa_stat waits for: an event of its own, so that neither
+// other streams nor a capture in another thread are touched.
+static exa_status launch_graph(exa_model *m, cudaGraphExec_t exec) {
+    CR(cudaGraphLaunch(exec, m->stream));
+    if (m->stamped) CR(cudaEventRecord(m->ev_done, m->stream));
+    return EXA_OK;
+}
+
 // exa_eval_all replays a CUDA graph of its launches (evaluation kernel plus the reductions it needs),
 // captured once per argument tuple on a private stream and cached (at most 4 tuples, least recently
 // used evicted).  When the model's stream is itself being captured, the launches go straight into
@@ -2857,8 +2871,7 @@ static exa_status eval_all_cached(exa_model *m, const double *x, const double *y
         if (ge.key == key) {
             ge.last_use = ++m->graph_clock;
             m->stamped = ge.stamped;
-            CR(cudaGraphLaunch(ge.exec, m->stream));
-            return EXA_OK;
+            return launch_graph(m, ge.exec);
         }
     if (!m->cap_stream) CR(cudaStreamCreateWithFlags(&m->cap_stream, cudaStreamNonBlocking));
     if (exa_status e = prepare_step(m)) return e;  // allocations cannot happen inside the capture
@@ -2898,8 +2911,7 @@ static exa_status eval_all_cached(exa_model *m, const double *x, const double *y
         m->graphs.erase(lru);
     }
     m->graphs.push_back({key, exec, ++m->graph_clock, m->stamped});
-    CR(cudaGraphLaunch(exec, m->stream));
-    return EXA_OK;
+    return launch_graph(m, exec);
 }
 
 exa_status exa_eval_all(exa_model *m, const double *x, const double *y, double sigma, double *f, double *g,
@@ -3205,14 +3217,19 @@ exa_status exa_stat(const exa_model *m, const char *key, double *value) {
     else if (k == "hprod_route") *value = m->hprod_how;
     else if (k == "eval_kernel_ms") {  // evaluation kernel(s) of the latest exa_eval_all step
         float ms = -1.0f;
-        unsigned long long t[2];
+        // (waiting on events and copying do not disturb captures in other threads in this mode)
+        cudaStreamCaptureMode mode = cudaStreamCaptureModeRelaxed;
+        cudaThreadExchangeStreamCaptureMode(&mode);
         if (m->stamped) {  // device timer (ns) around the kernel
-            if (cudaSetDevice(m->device) == cudaSuccess && cudaDeviceSynchronize() == cudaSuccess &&
-                cudaMemcpy(t, m->d_stamp, sizeof t, cudaMemcpyDeviceToHost) == cudaSuccess && t[1] >= t[0])
+            const unsigned long long *t = m->h_stamp;
+            if (cudaSetDevice(m->device) == cudaSuccess && cudaEventSynchronize(m->ev_done) == cudaSuccess &&
+                cudaMemcpyAsync(m->h_stamp, m->d_stamp, 2 * sizeof *t, cudaMemcpyDeviceToHost, m->cap_stream) == cudaSuccess &&
+                cudaStreamSynchronize(m->cap_stream) == cudaSuccess && t[1] >= t[0])
                 ms = (float)(1e-6 * (double)(t[1] - t[0]));
         } else if (!m->ev_k_valid || cudaEventSynchronize(m->ev_k1) != cudaSuccess ||
             cudaEventElapsedTime(&ms, m->ev_k0, m->ev_k1) != cudaSuccess)
             ms = -1.0f;
+        cudaThreadExchangeStreamCaptureMode(&mode);
         *value = ms;
     }
     else if (k == "eval_kernel_kind") {  // which generated kernel(s) the exa_eval_all step with every output runs

@@ -773,16 +773,7 @@ class Reduction {
             for (int i = 0; i < js->nj; i++) {
                 exa_red::Job &j = js->j[i];
                 j.blk0 = (int)blocks;
-                // wide: enough work for two blocks per SM at the larger share per thread
-                const i64 wide = 2 * 152;
-                switch (j.kind) {
-                case exa_red::PERM: j.wide = j.n >= wide * 2048; blocks += (j.n + (j.wide ? 2047 : 511)) / (j.wide ? 2048 : 512); break;
-                case exa_red::SEG: j.wide = j.n >= wide * 512; blocks += (j.n + (j.wide ? 511 : 255)) / (j.wide ? 512 : 256); break;
-                case exa_red::WSEG: case exa_red::CSUM: blocks += (j.n + 7) / 8; break;
-                case exa_red::CHUNK: case exa_red::BSEG: blocks += j.n; break;
-                case exa_red::OBJ: blocks += 1; break;
-                default: blocks += ((i64)(j.n + 31) / 32 - j.lo / 32 + 255) / 256; break;
-                }
+                blocks += exa_red::plan(j);
             }
             // A large launch mixes the sums (bound by the latency of dependent gathers) with the
             // streaming jobs, each in its own order; the sums first and alone otherwise.  The line:

@@ -76,6 +76,21 @@ constexpr int SHORT_MAX = 32;    // longest segment a single lane adds up
 // about 1.2 us for 4 entries per thread.  One 2000-entry variable of 2000 took a warp 42 us, a block 8.
 constexpr int WARP_MAX = 256, BLOCK_MAX = 8192;
 
+// Blocks of a job; decides `wide`: enough work for two blocks on each of 152 SMs at the larger share per thread.
+// In 64 bits: n reaches 2^31 - 1.
+inline long long plan(Job &j) {
+    const long long n = j.n, two = 2 * 152;
+    auto blocks = [n](long long per) { return (n + per - 1) / per; };
+    switch (j.kind) {
+    case PERM: j.wide = n >= two * 2048; return blocks(j.wide ? 2048 : 512);
+    case SEG: j.wide = n >= two * 512; return blocks(j.wide ? 512 : 256);
+    case WSEG: case CSUM: return blocks(8);
+    case CHUNK: case BSEG: return n;
+    case OBJ: return 1;
+    default: return ((n + 31) / 32 - j.lo / 32 + 255) / 256;
+    }
+}
+
 template <bool PROD>
 static __device__ __forceinline__ double entry(const Jobs &J, const double *src, int e) {
     if (!PROD) return __ldcg(src + e);

@@ -257,6 +257,7 @@ struct exa_model {
     std::vector<exa::Pattern> pats;
     std::vector<exa::Group> groups;
 
+    int sms = 0;  // of the device
     cudaLibrary_t lib = nullptr, lib_prod = nullptr;  // evaluation kernels; product kernels
     cudaKernel_t fn[exa::M_COUNT] = {};
     int regs[exa::M_COUNT] = {};
@@ -773,7 +774,7 @@ class Reduction {
             for (int i = 0; i < js->nj; i++) {
                 exa_red::Job &j = js->j[i];
                 j.blk0 = (int)blocks;
-                blocks += exa_red::plan(j);
+                blocks += exa_red::plan(j, m->sms);
             }
             // A large launch mixes the sums (bound by the latency of dependent gathers) with the
             // streaming jobs, each in its own order; the sums first and alone otherwise.  The line:
@@ -1429,15 +1430,13 @@ exa_status setup_kernels(exa_model *m, int block, int min_blocks = 0) {
 // starts about one wave of resident CTAs later.
 exa_status apply_grid(exa_model *m, int factor) {
     m->persist = factor;
-    int sms = 0;
-    CR(cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, m->device));
     for (int k = 0; k < exa::M_COUNT; k++) {
         m->grid[k] = m->ntiles[k];
         m->pfd[k] = 0;
         if (k == exa::M_STRUCT || exa::mode_prod(k)) continue;
         int occ = 0;
         CR(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, (const void *)m->fn[k], m->block, (size_t)m->dsmem[k]));
-        const long long wave = (long long)std::max(occ, 1) * sms;
+        const long long wave = (long long)std::max(occ, 1) * m->sms;
         const long long g = (long long)std::max(factor, 0) * wave;
         if (factor > 0 && g < m->ntiles[k]) m->grid[k] = (int)g;
         if (m->wave_pct > 0) {  // less than one wave: room on every SM for work on other streams
@@ -1450,7 +1449,7 @@ exa_status apply_grid(exa_model *m, int factor) {
 }
 
 // Models with fewer tiles (of 128 instances) than this are not tuned: four per SM.
-constexpr i64 TUNE_TILES = 4 * 152;
+i64 tune_tiles(const exa_model *m) { return 4 * (i64)m->sms; }
 i64 tiles_of_128(const exa_model *m) {
     i64 n = 0;
     for (const ExaPM &pm : m->h_pms) n += (pm.n_inst + 127) / 128;
@@ -1468,9 +1467,7 @@ i64 tiles_of_128(const exa_model *m) {
 // code-generator variants of a stage are compiled in parallel before they are timed.  Models too
 // small to fill the GPU are not tuned.
 exa_status autotune(exa_model *m) {
-    int sms = 0;
-    CR(cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, m->device));
-    if (tiles_of_128(m) < TUNE_TILES) return EXA_OK;
+    if (tiles_of_128(m) < tune_tiles(m)) return EXA_OK;
     Scratch S{m};
     double *x = nullptr, *y = nullptr, *part = nullptr;
     CR(S.get(&x, m->nvar));
@@ -2056,6 +2053,7 @@ exa_status create_impl(const exa_model_desc *const *descs, int nb, const exa_opt
     CR(dalloc(m, &m->d_theta, m->npar));
     CR(dalloc(m, &m->d_status, 1));
     CR(cudaMemset(m->d_status, 0, sizeof(int)));
+    CR(cudaDeviceGetAttribute(&m->sms, cudaDevAttrMultiProcessorCount, m->device));
     CR(dalloc(m, &m->d_stamp, 2));
     CR(cudaMallocHost((void **)&m->h_stamp, 2 * sizeof(unsigned long long)));
     CR(cudaEventCreateWithFlags(&m->ev_done, cudaEventDisableTiming));
@@ -2138,7 +2136,7 @@ exa_status create_impl(const exa_model_desc *const *descs, int nb, const exa_opt
     // 6000-bus 17.1 / 15.3 / 16.5, 20,000-step rocket 21.6 / 23.1 / 25.7.
     // FP64 only: another CTA size lets the compiler fuse other FP32 multiplies and adds, and mixed-precision
     // results would round differently.
-    if (!o.block_threads && m->precision == EXA_FP64 && tiles_of_128(m) < TUNE_TILES) m->block = 64;
+    if (!o.block_threads && m->precision == EXA_FP64 && tiles_of_128(m) < tune_tiles(m)) m->block = 64;
     if (exa_status e = setup_kernels(m, m->block, o.min_blocks)) return e;
 
     // structure pass on the device
@@ -2616,8 +2614,7 @@ static exa_status eval_all_chunked(exa_model *m, const double *x, const double *
 static exa_status build_step(exa_model *m, int i) {
     const Mode mode = i ? exa::M_ALL_B : exa::M_ALL;
     const int nb = m->nb;
-    int sms = 0, occ = 0;
-    CR(cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, m->device));
+    int occ = 0;
     CR(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, (const void *)m->fn_step[i], m->block, 0));
     const std::vector<ExaTile> &tiles = m->h_tiles[mode];
     std::vector<int> need(nb, 0);
@@ -2635,7 +2632,7 @@ static exa_status build_step(exa_model *m, int i) {
     };
     std::vector<ExaTask> items;
     items.reserve(tiles.size() + 64 * (size_t)nb);
-    const i64 grid_est = (i64)std::max(occ, 1) * sms;
+    const i64 grid_est = (i64)std::max(occ, 1) * m->sms;
     // items between a member's last tile and its reductions: two resident grids, or a quarter of
     // the tiles when there are few (so that small batches still interleave)
     const i64 lag = std::max<i64>(1, std::min<i64>(2 * grid_est, (i64)tiles.size() / 4));

@@ -76,10 +76,10 @@ constexpr int SHORT_MAX = 32;    // longest segment a single lane adds up
 // about 1.2 us for 4 entries per thread.  One 2000-entry variable of 2000 took a warp 42 us, a block 8.
 constexpr int WARP_MAX = 256, BLOCK_MAX = 8192;
 
-// Blocks of a job; decides `wide`: enough work for two blocks on each of 152 SMs at the larger share per thread.
+// Blocks of a job; decides `wide`: enough work for two blocks per SM at the larger share per thread.
 // In 64 bits: n reaches 2^31 - 1.
-inline long long plan(Job &j) {
-    const long long n = j.n, two = 2 * 152;
+inline long long plan(Job &j, int sms) {
+    const long long n = j.n, two = 2LL * sms;
     auto blocks = [n](long long per) { return (n + per - 1) / per; };
     switch (j.kind) {
     case PERM: j.wide = n >= two * 2048; return blocks(j.wide ? 2048 : 512);

@@ -2172,6 +2172,8 @@ exa_status create_impl(const exa_model_desc *const *descs, int nb, const exa_opt
         if (st) return fail(m, EXA_E_BOUNDS, "a resolved variable, parameter or row index is out of range");
     }
     if (exa_status e = build_structure(m)) return e;
+    dfree(m, &m->d_tvar, m->nnzt);  // (the variables are in the sums' lists now)
+    dfree(m, &m->d_uvar, m->nnzu);
     if (exa_status e = build_member_bounds(m)) return e;
     set_chunks(m, o.chunks ? o.chunks : 1);
     m->chunks_fixed = o.chunks != 0;

@@ -818,6 +818,21 @@ struct Scratch {
         if (e == cudaSuccess) mine.push_back(*p);
         return e;
     }
+    // four arrays of n, the same for every class of every gather-sum (a call per class cost more than its
+    // kernels: half of what the products had added to a 100,000-step rocket's creation)
+    cudaError_t classes(i64 n, int **a, int **b, int **c, int **d) {
+        if (n > class_n) {
+            if (cudaError_t e = get(&class_mem, 4 * n)) return e;
+            class_n = n;
+        }
+        *a = class_mem;
+        *b = *a + n;
+        *c = *b + n;
+        *d = *c + n;
+        return cudaSuccess;
+    }
+    int *class_mem = nullptr;
+    i64 class_n = 0;
 };
 
 // Key bits of an index below n (the radix sort makes one pass per eight).
@@ -877,10 +892,7 @@ exa_status build_ptr(exa_model *m, const unsigned long long *skeys, int shift, i
 exa_status build_seg_list(exa_model *m, Scratch &S, const int *ptr, const int *perm, const int *rows,
                           const unsigned *skip, int n, int lo, int hi, bool own_entries, SegList *L) {
     int *in = nullptr, *len = nullptr, *idx = nullptr, *cum = nullptr, *own = nullptr;
-    CR(S.get(&in, n));
-    CR(S.get(&len, n));
-    CR(S.get(&idx, n));
-    CR(S.get(&cum, n));
+    CR(S.classes(n, &in, &len, &idx, &cum));
     k_seg_class<<<grid_of(n, 256), 256, 0, m->stream>>>(ptr, rows, skip, n, lo, hi, in, len);
     CR(cudaGetLastError());
     CR(exa_inclusive_sum_i32(in, idx, n, m->stream));

@@ -227,9 +227,8 @@ struct SegList {
 // when it is built: elements with one entry or none are a plain gather over the codes `first`
 // (most CSC entries have one contributor, so most of the work is a permutation); short segments are
 // added up in ascending order by one lane, segments above SHORT_MAX entries by a warp, above WARP_MAX by
-// a block, and above BLOCK_MAX by blocks of CHUNK_LEN entries whose partial sums a second launch adds
-// up.  CSC sums are
-// `ordered`: every duplicate sum is short, i.e. in ascending COO order.
+// a block, and above BLOCK_MAX by blocks of CHUNK_LEN entries whose partial sums a second launch adds up.
+// CSC sums are `ordered`: one lane adds up every duplicate sum, however long, in ascending COO order.
 struct GatherSum {
     int longest = 0;        // entries of the longest segment
     int n = 0;              // positions of `first` (0: every element is in a list)

@@ -23,6 +23,7 @@
 #include <mutex>
 #include <thread>
 #include <string>
+#include <system_error>
 #include <vector>
 
 #include "exa_internal.h"
@@ -567,7 +568,7 @@ void dump_source(const std::string &src) {
 }
 
 // The cubins of the evaluation kernels' source and, when psrc is not null, of the product kernels'; what
-// is not in the cache is compiled at the same time.
+// is not in the cache is compiled at the same time, where the system gives a thread for it.
 exa_status cubins_of(exa_model *m, const std::string &src, const std::string *psrc,
                      std::shared_ptr<std::vector<char>> *cubin, std::shared_ptr<std::vector<char>> *pcubin) {
     exa_model scratch;
@@ -580,9 +581,13 @@ exa_status cubins_of(exa_model *m, const std::string &src, const std::string *ps
         }
     };
     std::thread th;
-    if (psrc) th = std::thread([&]() { pst = get(&scratch, *psrc, pcubin); });
+    try {
+        if (psrc) th = std::thread([&]() { pst = get(&scratch, *psrc, pcubin); });
+    } catch (const std::system_error &) {  // no thread to be had: one after the other
+    }
     st = get(m, src, cubin);
     if (th.joinable()) th.join();
+    else if (psrc) pst = get(&scratch, *psrc, pcubin);
     return st ? st : pst ? fail(m, pst, scratch.err) : EXA_OK;
 }
 

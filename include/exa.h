@@ -246,7 +246,7 @@ exa_status exa_set_stream(exa_model *m, void *stream);
 /* ------------------------------------------------------------------ callbacks (Sec. 2.1) */
 /* f[0] = f(x).  f: one device double.  Objective terms are reduced in FP64 in two stages (every
  * CTA sums the terms of all its tiles into one partial, then one ordered sum of the partials),
- * Sec. 7.2.3. */
+ * Sec. 7.2.3.  exa_eval_all adds the partials in another order: the last bits of the two f may differ. */
 exa_status exa_obj(exa_model *m, const double *x, double *f);
 
 /* f[0] = f(x), like exa_obj, but without the scratch buffer that exa_create allocates: the
@@ -298,7 +298,9 @@ exa_status exa_jac_csc_structure(const exa_model *m, int32_t *colptr, int32_t *r
                                  int32_t *coo2csc);
 exa_status exa_hess_csc_structure(const exa_model *m, int32_t *colptr, int32_t *rowval,
                                   int32_t *coo2csc);
-/* CSC values: the COO values of each (row, col) summed in ascending COO order. */
+/* CSC values: the COO values of each (row, col) summed in ascending COO order.  exa_hess_csc of FP64 models
+ * with compressed Hessian sums ("hess_compressed") differentiates each instance's weighted sum of patterns
+ * instead, so its values agree with those of exa_eval_all to rounding, not bit for bit. */
 exa_status exa_jac_csc(exa_model *m, const double *x, double *vals_csc);
 exa_status exa_hess_csc(exa_model *m, const double *x, const double *y, double sigma,
                         double *vals_csc);

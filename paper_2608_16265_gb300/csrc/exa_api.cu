@@ -1056,8 +1056,11 @@ void set_chunks(exa_model *m, int n) {
     m->chunk_b.push_back(nb);
 }
 
-// H v over the CSC values: the longest row or column that one lane walks.
-constexpr int HPROD_LANE_MAX = 256;
+// H v over the CSC values: the longest row or column that one lane walks.  100,000 rows of 24 variables times one
+// variable shared by L rows (longest row L + 23), us from the terms / by lanes, FP64: L = 16: 57 / 88, 32: 76 / 111;
+// mixed, sums by length / lanes: L = 1: 200 / 166, 4: 120 / 86, 8: 115 / 77, 16: 72 / 84, 32: 96 / 105; rocket of
+// 20,000 steps (80,004 entries in one row) 23 / 9579.
+constexpr int HPROD_LANE_MAX = 32;
 
 // Per-model structure: CSC of J and H, row groupings, gradient and augmentation segments.
 exa_status build_structure(exa_model *m) {

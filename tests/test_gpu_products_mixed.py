@@ -22,7 +22,7 @@ def shared_variable(n):
 
 MODELS = dict(rosenbrock=lambda: synth.rosenbrock(1500).flat, acopf=lambda: synth.acopf(300, 420, 50, seed=2).flat,
               goddard=lambda: synth.goddard(400).flat, **{f"shared{n}": (lambda n=n: shared_variable(n))
-                                                          for n in (1, 255, 256, 257, 8192, 8193, 20000)})
+                                                          for n in (1, 31, 32, 255, 256, 257, 8192, 8193, 20000)})
 
 
 @pytest.mark.parametrize("flags", [0, B.EXA_FLAG_LAZY_LOADS, B.EXA_FLAG_LAZY_LOADS | B.EXA_FLAG_SPLIT])
@@ -58,4 +58,4 @@ def test_products_of_the_entries(name, flags):
             ok = (np.abs(g - r) <= 2 * (cnt + 1) * 2.0 ** -53 * mag) & np.isfinite(mag)
         assert np.all(ok | (g == r) | (np.isnan(g) & np.isnan(r))), k
     rows = max(np.diff(cp).max(), np.bincount(hr).max())
-    assert int(m.stat("hprod_route")) == (2 if rows > 256 else 1)  # sums by length / one lane per variable
+    assert int(m.stat("hprod_route")) == (2 if rows > 32 else 1)  # sums by length / one lane per variable

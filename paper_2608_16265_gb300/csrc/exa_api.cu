@@ -244,6 +244,10 @@ struct GatherSum {
     std::vector<int> mb;            // first position of every batch member in `first`, or fill element
 };
 
+struct Slab {  // the free part of an allocation that small arrays share
+    char *at = nullptr, *end = nullptr;
+};
+
 struct exa_model {
     int device = 0;
     cudaStream_t stream = nullptr;
@@ -359,8 +363,7 @@ struct exa_model {
     // ... or two device timer stamps, in graphs of one evaluation kernel and its reductions
     unsigned long long *d_stamp = nullptr;
     bool stamped = false;  // the latest call used the stamps
-    cudaEvent_t ev_done = nullptr;            // the latest stamped call's end
-    unsigned long long *h_stamp = nullptr;    // page-locked copy for exa_stat
+    cudaEvent_t ev_done = nullptr;  // the latest stamped call's end
     bool grad_compact = false;
     int n_gseg = 0;
     int *d_gsegptr = nullptr, *d_gsegvar = nullptr;
@@ -378,6 +381,7 @@ struct exa_model {
            *d_cbuf = nullptr;
     std::vector<void *> allocs;
     size_t device_bytes = 0;
+    Slab slab;
     double nvrtc_ms = 0, create_ms = 0, tune_ms = 0;
     std::string err;
 };
@@ -396,17 +400,35 @@ exa_status fail(exa_model *m, exa_status s, const std::string &msg) {
     return s;
 }
 
+// Device memory that `owner` frees.  Small arrays (256-byte aligned) share allocations: a creation makes about
+// a hundred, and each call and its release cost more than such an array's kernels.
+cudaError_t device_alloc(Slab &s, std::vector<void *> &owner, void **p, size_t bytes) {
+    constexpr size_t SLAB = 256 << 10, SMALL = 32 << 10;
+    void *q = nullptr;
+    if (bytes > SMALL || (size_t)(s.end - s.at) < (bytes + 255) / 256 * 256) {
+        if (cudaError_t e = cudaMalloc(&q, bytes > SMALL ? bytes : SLAB)) return e;
+        owner.push_back(q);
+        if (bytes > SMALL) {
+            *p = q;
+            return cudaSuccess;
+        }
+        s.at = (char *)q;
+        s.end = s.at + SLAB;
+    }
+    *p = s.at;
+    s.at += (bytes + 255) / 256 * 256;
+    return cudaSuccess;
+}
+
 template <typename T>
 cudaError_t dalloc(exa_model *m, T **p, i64 count) {
     *p = nullptr;
     size_t bytes = (size_t)std::max<i64>(count, 1) * sizeof(T);
-    cudaError_t e = cudaMalloc((void **)p, bytes);
-    if (e == cudaSuccess) {
-        m->allocs.push_back(*p);
-        m->device_bytes += bytes;
-    }
+    cudaError_t e = device_alloc(m->slab, m->allocs, (void **)p, bytes);
+    if (e == cudaSuccess) m->device_bytes += bytes;
     return e;
 }
+// Gives an array back early (small ones go with the model).
 template <typename T>
 void dfree(exa_model *m, T **p, i64 count) {
     auto it = std::find(m->allocs.begin(), m->allocs.end(), (void *)*p);
@@ -432,8 +454,6 @@ void free_all(exa_model *m) {
     m->cap_stream = nullptr;
     if (m->side) cudaStreamDestroy(m->side);
     m->side = nullptr;
-    if (m->h_stamp) cudaFreeHost(m->h_stamp);
-    m->h_stamp = nullptr;
     for (cudaEvent_t *e : {&m->ev_join, &m->ev_first, &m->ev_done}) {
         if (*e) cudaEventDestroy(*e);
         *e = nullptr;
@@ -471,6 +491,7 @@ void free_all(exa_model *m) {
     }
     for (void *p : m->allocs) cudaFree(p);
     m->allocs.clear();
+    m->slab = Slab{};
     for (cudaLibrary_t *l : {&m->lib, &m->lib_prod}) {
         if (*l) cudaLibraryUnload(*l);
         *l = nullptr;
@@ -813,14 +834,13 @@ exa_status check_model(exa_model *m) {
 struct Scratch {
     exa_model *m;
     std::vector<void *> mine;
+    Slab slab{};
     ~Scratch() {
         for (void *p : mine) cudaFree(p);
     }
     template <typename T>
     cudaError_t get(T **p, i64 n) {
-        cudaError_t e = cudaMalloc((void **)p, (size_t)std::max<i64>(n, 1) * sizeof(T));
-        if (e == cudaSuccess) mine.push_back(*p);
-        return e;
+        return device_alloc(slab, mine, (void **)p, (size_t)std::max<i64>(n, 1) * sizeof(T));
     }
     // four arrays of n, the same for every class of every gather-sum (a call per class cost more than its
     // kernels: half of what the products had added to a 100,000-step rocket's creation)
@@ -2074,7 +2094,6 @@ exa_status create_impl(const exa_model_desc *const *descs, int nb, const exa_opt
     CR(cudaMemset(m->d_status, 0, sizeof(int)));
     CR(cudaDeviceGetAttribute(&m->sms, cudaDevAttrMultiProcessorCount, m->device));
     CR(dalloc(m, &m->d_stamp, 2));
-    CR(cudaMallocHost((void **)&m->h_stamp, 2 * sizeof(unsigned long long)));
     CR(cudaEventCreateWithFlags(&m->ev_done, cudaEventDisableTiming));
     std::vector<ExaPM> pms((size_t)nb * ng);
     for (int b = 0; b < nb; b++) {
@@ -3230,9 +3249,9 @@ exa_status exa_stat(const exa_model *m, const char *key, double *value) {
         cudaStreamCaptureMode mode = cudaStreamCaptureModeRelaxed;
         cudaThreadExchangeStreamCaptureMode(&mode);
         if (m->stamped) {  // device timer (ns) around the kernel
-            const unsigned long long *t = m->h_stamp;
+            unsigned long long t[2];
             if (cudaSetDevice(m->device) == cudaSuccess && cudaEventSynchronize(m->ev_done) == cudaSuccess &&
-                cudaMemcpyAsync(m->h_stamp, m->d_stamp, 2 * sizeof *t, cudaMemcpyDeviceToHost, m->cap_stream) == cudaSuccess &&
+                cudaMemcpyAsync(t, m->d_stamp, sizeof t, cudaMemcpyDeviceToHost, m->cap_stream) == cudaSuccess &&
                 cudaStreamSynchronize(m->cap_stream) == cudaSuccess && t[1] >= t[0])
                 ms = (float)(1e-6 * (double)(t[1] - t[0]));
         } else if (!m->ev_k_valid || cudaEventSynchronize(m->ev_k1) != cudaSuccess ||

@@ -2522,7 +2522,8 @@ exa_status exa_jac_csc(exa_model *m, const double *x, double *vals_csc) {
     // Without duplicates the CSC is a permutation: scattered by the evaluation kernel, except on large
     // models whose step gathers it (the tuner's choice), where the scattered 8-byte stores outlast the
     // arithmetic.  Scattered / gathered, us: 6.8 M entries (32 networks) 51 / 59, 24 M (PDE 2000^2 FP64,
-    // mixed) 141 / 156, 138 / 145; 52 M (256 networks) 486 / 369.
+    // mixed) 141 / 156, 138 / 145; 34 M (PDE 2400^2, 160 networks) 227 / 204, 312 / 239, mixed 222 / 206,
+    // 254 / 229; 47 M (PDE 2800^2) 315 / 273; 52 M (256 networks) 491 / 358, mixed 384 / 348.
     if (m->nnzj_csc == m->nnzj && (m->csc_direct || m->nnzj < (1 << 25))) {
         o.jac = nullptr;
         o.jcsc = vals_csc;
@@ -3079,7 +3080,7 @@ exa_status exa_eval_all_host(exa_model *m, const double *x, const double *y, dou
 // The products contract every instance's derivatives with the vector as they are formed (one term per
 // row, or per instance and variable of the fused group), so the Jacobian and Hessian values are neither
 // stored nor gathered; the terms of an augmented row or of a variable are then summed.  Bound by the
-// FP64 pipe (about 53, 52 and 70 operations per branch of a network, sin/cos included, at 528 G/s) and by
+// FP64 pipe (58, 60 and 69 operations per branch of a 30,000-bus network, all its patterns counted, at 528 G/s) and by
 // the gathers of x and of the vector.  Measured, the three together (before: all Jacobian and Hessian
 // values stored, then gathered per row, column and CSC entry): 30,000-bus network 107 -> 45 us, 32
 // networks (15.7 M entries) 313 -> 147 us, 100,000-step rocket 67.8 ms -> 129 us (one variable in

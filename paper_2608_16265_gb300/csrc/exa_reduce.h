@@ -12,11 +12,12 @@
 // Measured (GB300, whole exa_eval_all steps; before: one kernel per reduction on three streams, the
 // multi-entry CSC segments added onto a first pass): this alone took a 1000-variable model from 25.4 to
 // 15.4 us, a 30,000-bus network from 48.6 to 35.8, PDE 1000^2 from 94.6 to 80, PDE 2001^2 mixed from 307
-// to 274, the 256-network batch from 795 to 790 (with the later changes to the step's graph, the gradient
-// and the compressed sums: 12.3, 33.2, 72.7, 254 and 774 us).  On the batch the kernel takes 0.33 ms for
-// 52 M Jacobian and 24 M Hessian gathers: DRAM at 4.4 TB/s, the L1 tag stage near one line per clock (0.73
-// sectors per gathered value), so it gains from more gathers in flight only up to 48 warps x 8 per SM (64
-// warps: 808 us a step against 799; 40: 892; 4 or 16 gathers per thread at 48 warps: 825, 818).
+// to 274, the 256-network batch from 795 to 790 (with the later changes to the step's graph, the FP64
+// gradient and the FP64 compressed sums: 12.3, 33.2, 72.7, 273 and 774 us).  On the batch the kernel takes
+// 0.33 ms for 52 M Jacobian gathers and those of the Hessian sums; on its first 96 networks 121 us, 672 MB of
+// DRAM (5.6 TB/s, caches cold), 26.6 M sectors loaded, 66 % of the warps resident.  It gains from more gathers
+// in flight only up to 48 warps x 8 per SM (64 warps: 808 us a step against 799; 40: 892; 4 or 16 gathers per
+// thread at 48 warps: 825, 818).
 #pragma once
 
 #include <cuda_runtime.h>

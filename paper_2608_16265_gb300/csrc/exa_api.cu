@@ -400,15 +400,17 @@ exa_status fail(exa_model *m, exa_status s, const std::string &msg) {
     return s;
 }
 
+constexpr size_t SMALL_ARRAY = 32 << 10;  // bytes; up to here an array is a piece of a shared allocation
+
 // Device memory that `owner` frees.  Small arrays (256-byte aligned) share allocations: a creation makes about
 // a hundred, and each call and its release cost more than such an array's kernels.
 cudaError_t device_alloc(Slab &s, std::vector<void *> &owner, void **p, size_t bytes) {
-    constexpr size_t SLAB = 256 << 10, SMALL = 32 << 10;
+    constexpr size_t SLAB = 256 << 10;
     void *q = nullptr;
-    if (bytes > SMALL || (size_t)(s.end - s.at) < (bytes + 255) / 256 * 256) {
-        if (cudaError_t e = cudaMalloc(&q, bytes > SMALL ? bytes : SLAB)) return e;
+    if (bytes > SMALL_ARRAY || (size_t)(s.end - s.at) < (bytes + 255) / 256 * 256) {
+        if (cudaError_t e = cudaMalloc(&q, bytes > SMALL_ARRAY ? bytes : SLAB)) return e;
         owner.push_back(q);
-        if (bytes > SMALL) {
+        if (bytes > SMALL_ARRAY) {
             *p = q;
             return cudaSuccess;
         }
@@ -428,13 +430,15 @@ cudaError_t dalloc(exa_model *m, T **p, i64 count) {
     if (e == cudaSuccess) m->device_bytes += bytes;
     return e;
 }
-// Gives an array back early (small ones go with the model).
+// Gives an array of `count` elements back early.  Small ones go with the model: the first piece of a shared
+// allocation has the allocation's own address.
 template <typename T>
 void dfree(exa_model *m, T **p, i64 count) {
+    const size_t bytes = (size_t)std::max<i64>(count, 1) * sizeof(T);
     auto it = std::find(m->allocs.begin(), m->allocs.end(), (void *)*p);
-    if (it == m->allocs.end()) return;
+    if (bytes <= SMALL_ARRAY || !*p || it == m->allocs.end()) return;
     m->allocs.erase(it);
-    m->device_bytes -= (size_t)std::max<i64>(count, 1) * sizeof(T);
+    m->device_bytes -= bytes;
     cudaFree(*p);
     *p = nullptr;
 }

@@ -1080,6 +1080,13 @@ void set_chunks(exa_model *m, int n) {
     m->chunk_b.push_back(nb);
 }
 
+// What a dense gather-sum's lists no longer refer to: its segment starts, and its permutation when every
+// segment is short (short segments have entries of their own).
+void drop_unused(exa_model *m, const GatherSum &gs, int **ptr, i64 nseg, int **perm, i64 n) {
+    dfree(m, ptr, nseg + 1);
+    if (!gs.md.n && !gs.bl.n && !gs.lg.n) dfree(m, perm, n);
+}
+
 // H v over the CSC values: the longest row or column that one lane walks.  100,000 rows of 24 variables times one
 // variable shared by L rows (longest row L + 23), us from the terms / by lanes, FP64: L = 16: 57 / 88, 32: 76 / 111;
 // mixed, sums by length / lanes: L = 1: 200 / 166, 4: 120 / 86, 8: 115 / 77, 16: 72 / 84, 32: 96 / 105; rocket of
@@ -1212,8 +1219,9 @@ exa_status build_structure(exa_model *m) {
         }
         if (exa_status e = sort_with_perm(m, S, pk, n, bits_of(m->nvar), &skeys, perm)) return e;
         if (exa_status e = build_ptr(m, skeys, 0, n, m->nvar, &ptr)) return e;
-        if (exa_status e = build_gather_sum(m, S, ptr, perm, nullptr, (int)m->nvar, true, false, i ? &m->sum_u : &m->sum_t))
-            return e;
+        GatherSum &gs = i ? m->sum_u : m->sum_t;
+        if (exa_status e = build_gather_sum(m, S, ptr, perm, nullptr, (int)m->nvar, true, false, &gs)) return e;
+        drop_unused(m, gs, &ptr, m->nvar, &perm, n);
     }
     // ---- Jacobian entries by row (mixed; those by column follow the Jacobian CSC above)
     if (m->precision != EXA_FP64) {
@@ -1226,6 +1234,7 @@ exa_status build_structure(exa_model *m) {
         if (exa_status e = sort_with_perm(m, S, keys, nj, bits_of(m->ncon), &skeys, perm)) return e;
         if (exa_status e = build_ptr(m, skeys, 0, nj, m->ncon, &ptr)) return e;
         if (exa_status e = build_gather_sum(m, S, ptr, perm, nullptr, (int)m->ncon, true, false, &m->sum_r)) return e;
+        drop_unused(m, m->sum_r, &ptr, m->ncon, &perm, nj);
     }
     // ---- both mentions of every Hessian entry by variable
     if (m->hprod_how == exa_model::HPROD_ENTRIES) {
@@ -1241,6 +1250,7 @@ exa_status build_structure(exa_model *m) {
         if (exa_status e = sort_with_perm(m, S, pk, 2 * nc, bits_of(m->nvar + 1), &skeys, perm)) return e;
         if (exa_status e = build_ptr(m, skeys, 0, 2 * nc, m->nvar, &ptr)) return e;
         if (exa_status e = build_gather_sum(m, S, ptr, perm, nullptr, (int)m->nvar, true, false, &m->sum_u)) return e;
+        drop_unused(m, m->sum_u, &ptr, m->nvar, &perm, 2 * (i64)nc);
     }
 
     // ---- gradient segments by variable
